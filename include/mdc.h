@@ -224,7 +224,8 @@ int mdc_set_allreduce(mdc_handle h, mdc_allreduce_fn fn, void* ctx);
  * Tensor cores: with 16-bit, split or E4M3 storage, products of 8 or more columns run
  * on tensor cores only if the handle's operand buffers were reserved beforehand
  * (mdc_reserve(h, nv), which allocates, so call it at set-up); otherwise the product
- * runs on the slower SIMT path (correct, and counted by mdc_tc_fallback_count).
+ * runs on the slower SIMT path (correct, and counted by mdc_tc_fallback_count).  The same holds
+ * for complex64 storage from 5 columns on (not counted).
  * Arguments, layout, ownership and errors are otherwise those of mdc_forward.
  */
 #define MDC_STATIC_SCRATCH_COMPLEX (1 << 21)
@@ -418,7 +419,7 @@ int mdc_timing(mdc_handle h, int enable);
  * mdc_autotune -- choose, per direction and per column count (buckets 1, 2, 4, ... up to
  * ncol_max), the fastest per-frequency product variant for this handle by timing every variant
  * that can run on the handle's own buffers: the GEMV (up to 4 columns, or in passes over groups of
- * 4 up to 64 columns), the SIMT GEMM, and, for 16-bit and E4M3 storage, the tensor-core GEMM with
+ * 4 up to 64 columns), the float32 GEMM, and, for 16-bit and E4M3 storage, the tensor-core GEMM with
  * each column-tile width (32, 64, 128, 256).  Later
  * products use the variant of the smallest bucket holding their column count (the serving
  * engine still forces tensor cores so a job's arithmetic does not depend on its batch).  With
@@ -428,8 +429,9 @@ int mdc_timing(mdc_handle h, int enable);
  */
 int mdc_autotune(mdc_handle h, int ncol_max, void* stream);
 /* mdc_autotune_choice -- the variant selected for ncol columns: *path 0 = default rule, 1 = GEMV,
- * 2 = SIMT GEMM, 3 = tensor cores with column tile *bn, 4 = GEMV passes over groups of up to 4
- * columns. */
+ * 2 = float32 GEMM (complex64 storage: on tensor cores at float32 accuracy where the handle holds the
+ * operand buffers, else SIMT), 3 = tensor cores with column tile *bn, 4 = GEMV passes over groups of
+ * up to 4 columns. */
 int mdc_autotune_choice(mdc_handle h, int adjoint, int ncol, int* path, int* bn);
 
 /* mdc_set_option -- MDC_OPT_GRAPHS (value 1/0): when on, a marchenko_lsqr or

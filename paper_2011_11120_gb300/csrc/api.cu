@@ -280,6 +280,23 @@ int mdc::ensure_scratch(mdc_plan* p, int ncols) {
         p->tcSigma = sg;
         p->tc_cap = ncols;
     }
+    // complex64: the three-term operand of the tensor-core product.  It is three times the spectra, so
+    // it is taken only where it leaves the caller three quarters of the free memory; without it the
+    // products run on the GEMV / SIMT kernels.
+    if (p->storage == MDC_C64 && ncols >= C64_TC_MIN && ncols > p->tc_cap && ncols > p->tc_denied) {
+        const size_t bytes = tc_c64_scratch_elems(p, ncols) * 2;
+        size_t free_b = 0, total_b = 0;
+        void* b = nullptr;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4 &&
+            cudaMalloc(&b, bytes) == cudaSuccess) {
+            cudaFree(p->tcB);
+            p->tcB = b;
+            p->tc_cap = ncols;
+        } else {
+            cudaGetLastError();
+            p->tc_denied = ncols;
+        }
+    }
     return MDC_OK;
 }
 

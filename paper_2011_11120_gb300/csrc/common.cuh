@@ -142,9 +142,10 @@ struct mdc_plan {
     float2* specA = nullptr;    // [nf][max(nr,ns)][nv_cap]
     float2* specB = nullptr;
     // tensor-core path (FP16/BF16 storage): prepared B operand and its column scales
-    void* tcB = nullptr;        // [nf][rows_pad][max(2*ldg, nr8)] 16-bit
-    float* tcSigma = nullptr;   // [nf][tc_cap]
+    void* tcB = nullptr;        // [nf][rows_pad][max(2*ldg, nr8)] 16-bit; complex64: three planes [nf][2 ncol][..]
+    float* tcSigma = nullptr;   // [nf][tc_cap] (null for complex64)
     int tc_cap = 0;
+    int tc_denied = 0;          // complex64: columns whose operand did not fit (products run without it)
     int* err_flag = nullptr;    // device int: non-zero after a bounded device wait gave up
     unsigned long long wait_ns = 2000000000ull;   // bound on each tensor-core pipeline wait
     int64_t tc_fallbacks = 0;   // products the tensor-core rule chose that ran on another path
@@ -247,6 +248,16 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
 bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out,
                             int ldo, int voff_o, int ncol, cudaStream_t s, int path, int bn);
 size_t tc_scratch_elems(const mdc_plan* p, int ncol);
+
+// Tensor-core products of the complex64 copy (tc_c64.cu): float32 accuracy, from C64_TC_MIN columns on.
+// Products of 4 columns, GEMV / tensor cores (forward; adjoint): 0.90 / 0.65 and 0.54 / 0.65 ms on
+// 1681^2 x 150, 12 / 16 and 8 / 14 us on 81^2 x 40; of 5 columns, GEMV in two groups / tensor cores:
+// 1.43 / 0.65 and 1.04 / 0.65 ms, 20 / 16 and 12 / 14 us.
+constexpr int C64_TC_MIN = 5;
+bool tc_c64_ready(const mdc_plan* p, int ncol);        // operand buffers exist for ncol columns
+size_t tc_c64_scratch_elems(const mdc_plan* p, int ncol);
+bool launch_tc_c64(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out, int ldo,
+                   int voff_o, int ncol, cudaStream_t s, const int* active, bool scoped);
 
 // Quantise a complex64 kernel [nf][nr][ns] into the plan's reduced-storage copy and row scales.
 void launch_quantize(mdc_plan* p, const float2* G, const float* w, cudaStream_t s);

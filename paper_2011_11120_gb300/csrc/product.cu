@@ -11,8 +11,9 @@
 //            one frequency, each warp walks a subset of rows r reading the 512-byte
 //            row segment, and the per-warp partial sums meet in shared memory.
 //            No atomics, no second copy of G.
-// Many columns (GEMM regime): a tiled FP32 complex GEMM (64x64 complex tile per
-// CTA, 4x4 per thread), the adjoint tile loader conjugating and transposing.
+// Many columns (GEMM regime): tensor cores (tc_c64.cu, tc_gemm.cu); where a handle has no
+// operand buffers for them, a tiled FP32 complex GEMM (64x64 complex tile per CTA, 4x4 per
+// thread), the adjoint tile loader conjugating and transposing.
 #include "common.cuh"
 #include <cstdlib>
 
@@ -905,6 +906,8 @@ bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi
     if (path == PATH_TC)
         return storage_tc(p->storage) && p->tcB && ncol <= p->tc_cap &&
                launch_tc_product(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, bn);
+    if (path == PATH_SIMT && tc_c64_ready(p, ncol))
+        return launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, false);
     return product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, path);
 }
 
@@ -933,6 +936,10 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
         path = PATH_AUTO;
     }
     if (tc_wanted) ++p->tc_fallbacks;
+    // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand buffers exist
+    if ((path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN)) && tc_c64_ready(p, ncol) &&
+        launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, true))
+        return;
     LaunchScope ls(p, s, adjoint ? MDC_KC_PRODUCT_ADJ : MDC_KC_PRODUCT_FWD);
     if (!product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, path))
         product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, PATH_AUTO);

@@ -1,0 +1,75 @@
+"""Complex64 products on tensor cores (five columns or more): parity with the FP64 oracle at the edges
+of the kernel's tiles, and the bounded waits.
+
+Tolerance: each output sums at most 32 chunk sums per group in float32 (RMS rounding 2^-24 / sqrt(3) per
+addition against partial sums that grow like a random walk: sqrt(32 / 2) 2^-24 / sqrt(3) = 1.4e-7), each
+chunk truncated at most four times by 2^-25 of its size (1.2e-7), between two transforms of about
+1.2e-7 each: 2.6e-7 together, and four times that for structure in the data.
+"""
+import numpy as np
+import pytest
+
+from oracle import mdc as omdc
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+
+# (nr, ns, nf, nv): column tiles of 32, 64, 96 and 128 real columns with remainders and more than one
+# tile; row tiles of 128 kernel rows (64 columns, adjoint) exact, one over, one under; reduction steps of
+# 32 reals exact and with a tail, one step, and more than one group of 64 steps in either direction
+CASES = [(1, 7, 3, 5), (129, 65, 9, 16), (128, 64, 5, 17), (127, 63, 5, 32), (77, 1100, 6, 33),
+         (2100, 40, 5, 48), (130, 129, 4, 49), (64, 50, 4, 64), (33, 300, 4, 65), (200, 31, 3, 130)]
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def problem(nr, ns, nf, nv, nt=64):
+    rng = np.random.default_rng(nr + 7 * ns + 31 * nv)
+    G = (rng.standard_normal((nf, nr, ns)) + 1j * rng.standard_normal((nf, nr, ns))) / np.sqrt(ns)
+    G = G.astype(np.complex64)
+    x = rng.standard_normal((nt, ns, nv)).astype(np.float32)
+    y = rng.standard_normal((nt, nr, nv)).astype(np.float32)
+    return G, x, y
+
+
+@pytest.mark.parametrize("nr,ns,nf,nv", CASES)
+def test_c64_tensor_core_products_match_oracle(nr, ns, nf, nv):
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(nr, ns, nf, nv)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    m.mdc_timing(op.h, True)
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    assert m.mdc_timing_read(op.h, "tc_prep")[1] == 2          # both products ran on tensor cores
+    yc = op.forward(torch.from_numpy(x).cuda(), conj=True).cpu().numpy()
+    m.mdc_device_status(op.h)
+    op.close()
+    G = G.astype(np.complex128)
+    assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
+    assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
+    assert rel(yc, omdc.forward_conj_kernel(G, x, 0.004, 400.0)) <= TOL
+
+
+def test_c64_tensor_core_wait_limit():
+    """A limit the pipeline cannot meet is reported, and the handle works again with the default one."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(300, 1100, 20, 16)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    xt = torch.from_numpy(x).cuda()
+    op.forward(xt)
+    m.mdc_device_status(op.h)
+    m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, 1)
+    for _ in range(20):
+        op.forward(xt)
+    with pytest.raises(m.MDCError) as e:
+        m.mdc_device_status(op.h)
+    assert e.value.status == -4
+    m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, 0)
+    yg = op.forward(xt).cpu().numpy()
+    m.mdc_device_status(op.h)
+    op.close()
+    assert rel(yg, omdc.forward(G.astype(np.complex128), x, 0.004, 400.0)) <= TOL
