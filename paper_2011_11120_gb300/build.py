@@ -33,7 +33,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
            "-Xptxas", "-v"] + ARCH
 
-SOURCES = ["api.cu", "fft.cu", "product.cu", "lsqr.cu", "static_scratch.cu", "mdd.cu", "tc_gemm.cu", "tc_c64.cu"]
+SOURCES = ["api.cu", "fft.cu", "fft_inv_small.cu", "fft_inv_512.cu", "fft_inv_1024.cu",
+           "product.cu", "lsqr.cu", "static_scratch.cu", "mdd.cu", "tc_gemm.cu", "tc_c64.cu"]
 
 
 def nvcc() -> str:

@@ -183,7 +183,7 @@ struct RfftArgs {
     int ldv, voff;
     const float2* tw;
     const int* active;     // if non-null and *active == 0 the kernel does nothing
-    int vec4;              // set by the launcher: x (and x2) 16-byte aligned rows, C % 4 == 0
+    int v2;                // set by the launcher: C even, x (and x2) 8-byte aligned
     int* err;              // set by the launcher: the plan's device error flag (bounds checks)
 };
 struct IrfftArgs {
@@ -250,8 +250,8 @@ bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi
 size_t tc_scratch_elems(const mdc_plan* p, int ncol);
 
 // Tensor-core products of the complex64 copy (tc_c64.cu): float32 accuracy, from C64_TC_MIN columns on.
-// Products of 4 columns, GEMV / tensor cores (forward; adjoint): 0.90 / 0.65 and 0.54 / 0.65 ms on
-// 1681^2 x 150, 12 / 16 and 8 / 14 us on 81^2 x 40; of 5 columns, GEMV in two groups / tensor cores:
+// Products of 4 columns, GEMV / tensor cores (forward; adjoint): 0.59 / 0.65 and 0.54 / 0.65 ms on
+// 1681^2 x 150, 10 / 16 and 8 / 14 us on 81^2 x 40; of 5 columns, GEMV in two groups / tensor cores:
 // 1.43 / 0.65 and 1.04 / 0.65 ms, 20 / 16 and 12 / 14 us.
 constexpr int C64_TC_MIN = 5;
 bool tc_c64_ready(const mdc_plan* p, int ncol);        // operand buffers exist for ncol columns

@@ -15,12 +15,10 @@
 // back, and reads column A from the real and column B from the imaginary part.
 //
 // Twiddles come from a float64 host table rounded once to float32.
-#include "common.cuh"
+#include "fft_common.cuh"
 
 namespace mdc {
 namespace {
-
-constexpr int FFT_THREADS = 256;
 
 __device__ __forceinline__ int bitrev(int v, int logn) { return (int)(__brev((unsigned)v) >> (32 - logn)); }
 
@@ -160,193 +158,6 @@ __global__ void __launch_bounds__(FFT_THREADS) irfft_kernel(IrfftArgs a, int log
     }
 }
 
-// ------------------------------------------------------------------ four-step kernels
-// nt = N1 * N2 (N1, N2 in {8, 16, 32}).  Pass A: for each residue n2, an N1-point DFT in
-// registers over t = n1 * N2 + n2, then the twiddle W_nt^(n2 k1); pass B: for each k1 an
-// N2-point DFT over the N2 consecutive rows k1 * N2 + n2.  Result bin k = k1 + N1 * k2
-// sits in row k1 * N2 + k2.  Four shared-memory sweeps per transform instead of
-// 2 log2(nt) + 1 for radix 2.  Layout: row t of P complex sequences at
-// t * RS + (t / N2) * BP, RS = P + 1 and BP chosen so that both passes spread a warp's
-// 8-byte accesses over distinct bank pairs.
-
-__host__ __device__ constexpr int brev_bits(int i, int bits) {
-    int r = 0;
-    for (int b = 0; b < bits; ++b) r |= ((i >> b) & 1) << (bits - 1 - b);
-    return r;
-}
-__host__ __device__ constexpr int clog2(int n) { return n <= 1 ? 0 : 1 + clog2(n / 2); }
-
-// Roots of unity as compile-time constants: cos and sin of 2*pi/R from the half-angle identities
-// (cos(t/2) = sqrt((1 + cos t) / 2), sin(t/2) = sin t / (2 cos(t/2))) starting at t = pi/2, then
-// powers by angle addition, all in double precision and rounded once to float.
-struct Rot {
-    double c, s;
-};
-constexpr double newton_sqrt(double x) {
-    double r = x > 1.0 ? x : 1.0;
-    for (int i = 0; i < 64; ++i) r = 0.5 * (r + x / r);
-    return r;
-}
-constexpr Rot unit_root(int R, int m) {   // exp(+2 pi i m / R)
-    Rot b{0.0, 1.0};
-    if (R == 1) b = Rot{1.0, 0.0};
-    if (R == 2) b = Rot{-1.0, 0.0};
-    for (int r = 4; r < R; r *= 2) {
-        const double c = newton_sqrt(0.5 * (1.0 + b.c));
-        b = Rot{c, b.s / (2.0 * c)};
-    }
-    Rot w{1.0, 0.0};
-    for (int i = 0; i < m; ++i) w = Rot{w.c * b.c - w.s * b.s, w.s * b.c + w.c * b.s};
-    return w;
-}
-
-// exp(-2 pi i m / 32) for m < 16: every twiddle of the in-register DFTs (R <= 32) is one of
-// these; as constant-bank operands they need no load.
-#define MDC_ROOT32(m) float2{(float)unit_root(32, m).c, -(float)unit_root(32, m).s}
-__constant__ float2 kRoot32[16] = {
-    MDC_ROOT32(0),  MDC_ROOT32(1),  MDC_ROOT32(2),  MDC_ROOT32(3),  MDC_ROOT32(4),  MDC_ROOT32(5),
-    MDC_ROOT32(6),  MDC_ROOT32(7),  MDC_ROOT32(8),  MDC_ROOT32(9),  MDC_ROOT32(10), MDC_ROOT32(11),
-    MDC_ROOT32(12), MDC_ROOT32(13), MDC_ROOT32(14), MDC_ROOT32(15)};
-#undef MDC_ROOT32
-
-// Complex add and subtract as one packed two-lane float32 instruction (sm_100 and later);
-// each lane rounds to nearest like the scalar operation.
-__device__ __forceinline__ float2 padd(float2 a, float2 b) {
-    float2 r;
-    asm("{.reg .b64 pa, pb, pr;\n\t"
-        "mov.b64 pa, {%2, %3};\n\t"
-        "mov.b64 pb, {%4, %5};\n\t"
-        "add.rn.f32x2 pr, pa, pb;\n\t"
-        "mov.b64 {%0, %1}, pr;}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ float2 psub(float2 a, float2 b) {
-    float2 r;
-    asm("{.reg .b64 pa, pb, pr;\n\t"
-        "mov.b64 pa, {%2, %3};\n\t"
-        "mov.b64 pb, {%4, %5};\n\t"
-        "sub.rn.f32x2 pr, pa, pb;\n\t"
-        "mov.b64 {%0, %1}, pr;}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-
-// Length-R DFT (R <= 32) of a register array, forward sign exp(-2 pi i n k / R) or, with INV,
-// the inverse sign (unscaled): decimation in frequency (natural order in, bit-reversed order
-// out), then a compile-time permutation back to natural order.  After unrolling every index
-// and twiddle choice is a constant: quarter turns are a swap, eighth turns take the
-// equal-magnitude short form, the rest multiply by a table constant.
-template <int R, bool INV>
-__device__ __forceinline__ void reg_fft(float2 (&a)[R]) {
-    static_assert(R <= 32, "register DFT length");
-    constexpr int L = clog2(R);
-    constexpr float h8 = (float)unit_root(8, 1).c;
-#pragma unroll
-    for (int st = 0; st < L; ++st) {
-        const int h = R >> (st + 1);          // half span of this stage
-#pragma unroll
-        for (int g = 0; g < R; g += 2 * h) {
-#pragma unroll
-            for (int j = 0; j < h; ++j) {
-                const float2 u = a[g + j], v = a[g + j + h];
-                a[g + j] = padd(u, v);
-                float2 d = psub(u, v);
-                const int m = j << st;       // twiddle exp(-+2 pi i m / R)
-                if (m == 0) {
-                } else if (4 * m == R) {
-                    d = INV ? make_float2(-d.y, d.x) : make_float2(d.y, -d.x);
-                } else if (8 * m == R) {
-                    d = INV ? make_float2(h8 * (d.x - d.y), h8 * (d.x + d.y))
-                            : make_float2(h8 * (d.x + d.y), h8 * (d.y - d.x));
-                } else if (8 * m == 3 * R) {
-                    d = INV ? make_float2(-h8 * (d.x + d.y), h8 * (d.x - d.y))
-                            : make_float2(h8 * (d.y - d.x), -h8 * (d.x + d.y));
-                } else {
-                    const float2 w = kRoot32[m * (32 / R)];
-                    d = cmul(d, INV ? cconj(w) : w);
-                }
-                a[g + j + h] = d;
-            }
-        }
-    }
-    float2 b[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) b[i] = a[brev_bits(i, L)];
-#pragma unroll
-    for (int i = 0; i < R; ++i) a[i] = b[i];
-}
-
-// PP: complex sequences per CTA, or 0 for the default of about 8192 complex values per tile (the
-// few-column variant PP = max(1024 / NT, 2) spreads small batches over more CTAs).
-template <int N1, int N2, int PP = 0> struct FourStep {
-    static constexpr int NT = N1 * N2;
-    static constexpr int P0 = 8192 / NT;
-    static constexpr int P = PP ? PP : (P0 > 32 ? 32 : (P0 < 8 ? 8 : P0));   // complex sequences per CTA
-    static constexpr int CT = 2 * P;                                  // real columns per CTA
-    // Rows of P complex values, unpadded, plus BP slots after every block of N2 rows: with P = 8
-    // two consecutive rows (or blocks, in pass B) then fill all 16 bank pairs, and rows stay
-    // 16-byte aligned for vector accesses.
-    static constexpr int RS = P;
-    static constexpr int BP = P == 8 ? 8 : 0;
-    static constexpr int ZSIZE = NT * RS + N1 * BP;                  // float2 elements
-    // twiddle table and tile; the inverse transform's column-sum reduction reuses the tile
-    static constexpr size_t smem = (size_t)(NT / 2 + ZSIZE) * sizeof(float2);
-    static constexpr size_t smem_full = (size_t)(NT + ZSIZE) * sizeof(float2);   // full-period twiddles
-    static_assert(ZSIZE * sizeof(float2) >= FFT_THREADS * 4 * sizeof(double), "reduction fits the tile");
-    __device__ static __forceinline__ int zi(int t, int j) { return t * RS + (t / N2) * BP + j; }
-};
-
-__device__ __forceinline__ float2 tw_full(const float2* tw, int m, int nt) {
-    return m < (nt >> 1) ? tw[m] : make_float2(-tw[m - (nt >> 1)].x, -tw[m - (nt >> 1)].y);
-}
-
-// Second pass of the four-step transform: the length-N2 DFTs over n2 of every block k1, in
-// place; ends with a barrier.
-template <int N1, int N2, bool INV, int PP = 0>
-__device__ __forceinline__ void four_step_pass_b(float2* z) {
-    using F = FourStep<N1, N2, PP>;
-    constexpr int P = F::P;
-    for (int task = threadIdx.x; task < P * N1; task += FFT_THREADS) {
-        const int j = task % P, k1 = task / P;
-        float2 r[N2];
-#pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) r[n2] = z[F::zi(k1 * N2 + n2, j)];
-        reg_fft<N2, INV>(r);
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) z[F::zi(k1 * N2 + k2, j)] = r[k2];
-    }
-    __syncthreads();
-}
-
-// tw: the twiddle table W_NT^m of the transform's sign (conjugated for INV), m < NT/2, or with
-// FULL the whole period m < NT (no sign select per twiddle).
-template <int N1, int N2, bool INV, bool FULL = false, int PP = 0>
-__device__ __forceinline__ void four_step(float2* z, const float2* tw) {
-    using F = FourStep<N1, N2, PP>;
-    constexpr int P = F::P;
-    for (int task = threadIdx.x; task < P * N2; task += FFT_THREADS) {
-        const int j = task % P, n2 = task / P;
-        float2 r[N1];
-#pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) r[n1] = z[F::zi(n1 * N2 + n2, j)];
-        reg_fft<N1, INV>(r);
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) {
-            const float2 v = k1 == 0 ? r[0] : cmul(r[k1], FULL ? tw[n2 * k1] : tw_full(tw, n2 * k1, F::NT));
-            z[F::zi(k1 * N2 + n2, j)] = v;
-        }
-    }
-    __syncthreads();
-    four_step_pass_b<N1, N2, INV, PP>(z);
-}
-
-// Row holding bin (or time sample) q after four_step.
-template <int N1, int N2>
-__device__ __forceinline__ int out_row(int q) { return (q % N1) * N2 + q / N1; }
-
 // WIN: the window Theta multiplies the input; X2: a second input is added.  The input scale is
 // applied to the separated spectrum (the transform is linear), together with its factor 1/2.
 template <int N1, int N2, bool WIN, bool X2, int PP>
@@ -363,81 +174,61 @@ __global__ void __launch_bounds__(FFT_THREADS, 2) rfft4_kernel(RfftArgs a) {
         tw[i] = w;
         tw[i + NT / 2] = make_float2(-w.x, -w.y);
     }
-    // Load the [NT][CT] tile with many independent loads in flight per thread.
-    auto put = [&](int t, int cl, float v) {
-        if constexpr (WIN) {
-            const int tau = t < (NT >> 1) ? t : NT - t;
-            if (tau >= *MDC_AT(a.cut, c0 + cl, 1, a.C, a.err, 11)) v = 0.f;
-        }
-        reinterpret_cast<float*>(z + F::zi(t, cl >> 1))[cl & 1] = v;
-    };
-    if (a.vec4 && c0 + CT <= a.C) {
-        // First pass straight from global memory: task (j, n2) loads the column pair
-        // (c0 + 2j, c0 + 2j + 1) at rows n1 * N2 + n2 (a warp reads whole 64- or 128-byte row
-        // segments), applies window and scale, transforms over n1 in registers, twiddles, and
-        // writes the tile; only the second pass goes through shared memory.
-        __syncthreads();                                  // twiddle table
-        constexpr int P = F::P;
-        const size_t rstride = (size_t)N2 * a.C;          // floats between the rows n1 and n1 + 1
-        for (int task = threadIdx.x; task < P * N2; task += FFT_THREADS) {
-            const int j = task % P, n2 = task / P, c = c0 + 2 * j;
-            const size_t xo = c + (size_t)n2 * a.C;
-            float2 r[N1];
+    // First pass straight from global memory: task (j, n2) loads the column pair (c0 + 2j, c0 + 2j + 1)
+    // at rows n1 * N2 + n2 (a warp reads whole 64- or 128-byte row segments), applies the window,
+    // transforms over n1 in registers, twiddles, and writes the tile; only the second pass goes through
+    // shared memory.  Columns of odd count or alignment are read one by one.
+    __syncthreads();                                      // twiddle table
+    constexpr int P = F::P;
+    const bool pairs = a.v2 && c0 + CT <= a.C;
+    const size_t rstride = (size_t)N2 * a.C;              // floats between the rows n1 and n1 + 1
+    [[maybe_unused]] const long long nx = (long long)NT * a.C;
+    for (int task = threadIdx.x; task < P * N2; task += FFT_THREADS) {
+        const int j = task % P, n2 = task / P, c = c0 + 2 * j;
+        const bool has0 = c < a.C, has1 = c + 1 < a.C;
+        const size_t xo = c + (size_t)n2 * a.C;
+        float2 r[N1];
+        if (pairs) {
 #pragma unroll
             for (int n1 = 0; n1 < N1; ++n1)
-                r[n1] = *reinterpret_cast<const float2*>(MDC_AT(a.x, xo + n1 * rstride, 2, (long long)NT * a.C, a.err, 12));
-            if constexpr (X2) {
+                r[n1] = *reinterpret_cast<const float2*>(MDC_AT(a.x, xo + n1 * rstride, 2, nx, a.err, 12));
+        } else {
 #pragma unroll
-                for (int n1 = 0; n1 < N1; ++n1) {
-                    const float2 w = *reinterpret_cast<const float2*>(MDC_AT(a.x2, xo + n1 * rstride, 2, (long long)NT * a.C, a.err, 13));
-                    r[n1].x += w.x;
-                    r[n1].y += w.y;
-                }
-            }
-            if constexpr (WIN) {
-                const int cut0 = *MDC_AT(a.cut, c, 1, a.C, a.err, 14), cut1 = *MDC_AT(a.cut, c + 1, 1, a.C, a.err, 14);
-#pragma unroll
-                for (int n1 = 0; n1 < N1; ++n1) {
-                    const int t = n1 * N2 + n2;
-                    const int tau = t < (NT >> 1) ? t : NT - t;
-                    if (tau >= cut0) r[n1].x = 0.f;
-                    if (tau >= cut1) r[n1].y = 0.f;
-                }
-            }
-            reg_fft<N1, false>(r);
-#pragma unroll
-            for (int k1 = 0; k1 < N1; ++k1)
-                z[F::zi(k1 * N2 + n2, j)] = k1 == 0 ? r[0] : cmul(r[k1], tw[n2 * k1]);
+            for (int n1 = 0; n1 < N1; ++n1)
+                r[n1] = make_float2(has0 ? *MDC_AT(a.x, xo + n1 * rstride, 1, nx, a.err, 12) : 0.f,
+                                    has1 ? *MDC_AT(a.x, xo + n1 * rstride + 1, 1, nx, a.err, 12) : 0.f);
         }
-        __syncthreads();
-        four_step_pass_b<N1, N2, false, PP>(z);
-    } else {
-        constexpr int PER = NT * CT / FFT_THREADS, B = PER < 16 ? PER : 16;
-#pragma unroll 1
-        for (int b0 = 0; b0 < PER; b0 += B) {
-            float v[B];
+        if constexpr (X2) {
 #pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int idx = threadIdx.x + (b0 + u) * FFT_THREADS;
-                const int t = idx / CT, c = c0 + idx % CT;
-                v[u] = 0.f;
-                if (c < a.C) {
-                    const size_t off = (size_t)t * a.C + c;
-                    v[u] = *MDC_AT(a.x, off, 1, (long long)NT * a.C, a.err, 15);
-                    if constexpr (X2) v[u] += *MDC_AT(a.x2, off, 1, (long long)NT * a.C, a.err, 16);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int idx = threadIdx.x + (b0 + u) * FFT_THREADS;
-                const int t = idx / CT, cl = idx % CT;
-                if (c0 + cl < a.C) put(t, cl, v[u]);
-                else reinterpret_cast<float*>(z + F::zi(t, cl >> 1))[cl & 1] = 0.f;
+            for (int n1 = 0; n1 < N1; ++n1) {
+                float2 w;
+                if (pairs)
+                    w = *reinterpret_cast<const float2*>(MDC_AT(a.x2, xo + n1 * rstride, 2, nx, a.err, 13));
+                else
+                    w = make_float2(has0 ? *MDC_AT(a.x2, xo + n1 * rstride, 1, nx, a.err, 13) : 0.f,
+                                    has1 ? *MDC_AT(a.x2, xo + n1 * rstride + 1, 1, nx, a.err, 13) : 0.f);
+                r[n1].x += w.x;
+                r[n1].y += w.y;
             }
         }
-        __syncthreads();
-        four_step<N1, N2, false, true, PP>(z, tw);
+        if constexpr (WIN) {
+            const int cut0 = has0 ? *MDC_AT(a.cut, c, 1, a.C, a.err, 14) : 0;
+            const int cut1 = has1 ? *MDC_AT(a.cut, c + 1, 1, a.C, a.err, 14) : 0;
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) {
+                const int t = n1 * N2 + n2;
+                const int tau = t < (NT >> 1) ? t : NT - t;
+                if (tau >= cut0) r[n1].x = 0.f;
+                if (tau >= cut1) r[n1].y = 0.f;
+            }
+        }
+        reg_fft<N1, false>(r);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1)
+            z[F::zi(k1 * N2 + n2, j)] = k1 == 0 ? r[0] : cmul(r[k1], tw[n2 * k1]);
     }
+    __syncthreads();
+    four_step_pass_b<N1, N2, false, PP>(z);
     const float hs = 0.5f * coef(a.scale);
     // Bin k = k1 + N1 * k2 sits in row k1 * N2 + k2, its mirror NT - k in row
     // ((-k1) mod N1) * N2 + (NT/N1 - k2 - [k1 > 0]) (k > 0).  A thread keeps one column and walks
@@ -473,324 +264,6 @@ __global__ void __launch_bounds__(FFT_THREADS, 2) rfft4_kernel(RfftArgs a) {
                 if (a.conj) r.y = -r.y;
                 *MDC_AT(a.X, dsto + (size_t)(k - a.k0) * kstride, 1, (long long)a.nf * a.S * a.ldv, a.err, 17) = r;
             }
-        }
-    }
-}
-
-// Forward transform of the tile the inverse kernel leaves behind: storage row rho = t1 * N2 + t2
-// holds time t = t1 + N1 t2 of P packed column pairs.  With k = k2 + N2 k1,
-//   X[k] = sum_t1 W_N1^(t1 k1) [ W_NT^(t1 k2) sum_t2 W_N2^(t2 k2) x[t1 + N1 t2] ],
-// so N2-point DFTs in each block t1, the twiddle, then N1-point DFTs over t1 leave bin k in row
-// k1 * N2 + k2 = k (natural order).  The two columns of each pair are then separated as in the
-// forward kernels (scale 1/2, optional conjugation) and bins [k0, k0 + nf) stored into fwd_X.
-// tw: the inverse transform's half-period table, conjugated here.
-template <int N1, int N2, int PP>
-__device__ __forceinline__ void fused_forward(const IrfftArgs& a, float2* z, const float2* tw, int c0) {
-    using F = FourStep<N1, N2, PP>;
-    constexpr int NT = F::NT, CT = F::CT, P = F::P;
-    for (int task = threadIdx.x; task < P * N1; task += FFT_THREADS) {
-        const int j = task % P, t1 = task / P;
-        float2 r[N2];
-#pragma unroll
-        for (int t2 = 0; t2 < N2; ++t2) r[t2] = z[F::zi(t1 * N2 + t2, j)];
-        reg_fft<N2, false>(r);
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2)
-            z[F::zi(t1 * N2 + k2, j)] = k2 == 0 ? r[0] : cmul(r[k2], cconj(tw_full(tw, t1 * k2, NT)));
-    }
-    __syncthreads();
-    for (int task = threadIdx.x; task < P * N2; task += FFT_THREADS) {
-        const int j = task % P, k2 = task / P;
-        float2 r[N1];
-#pragma unroll
-        for (int t1 = 0; t1 < N1; ++t1) r[t1] = z[F::zi(t1 * N2 + k2, j)];
-        reg_fft<N1, false>(r);
-#pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) z[F::zi(k1 * N2 + k2, j)] = r[k1];
-    }
-    __syncthreads();
-    constexpr int G = FFT_THREADS / CT;
-    const int cl = threadIdx.x % CT, g = threadIdx.x / CT, c = c0 + cl;
-    if (c >= a.C) return;
-    int s, v;
-    if ((a.nv % CT) == 0) {
-        s = c0 / a.nv;
-        v = c0 - s * a.nv + cl;
-    } else {
-        s = c / a.nv;
-        v = c - s * a.nv;
-    }
-    const size_t dsto = (size_t)s * a.ldv + a.fwd_voff + v;
-    const size_t kstride = (size_t)a.S * a.ldv;
-    const int j = cl >> 1;
-    const bool odd = (cl & 1) != 0;
-    for (int kk = g; kk < a.nf; kk += G) {
-        const int k = a.k0 + kk;
-        const float2 Z = z[F::zi(k, j)];
-        const float2 Zm = k == 0 ? Z : z[F::zi(NT - k, j)];
-        float2 r = odd ? make_float2(0.5f * (Z.y + Zm.y), 0.5f * (Zm.x - Z.x))
-                       : make_float2(0.5f * (Z.x + Zm.x), 0.5f * (Z.y - Zm.y));
-        if (a.fwd_conj) r.y = -r.y;
-        *MDC_AT(a.fwd_X, dsto + (size_t)kk * kstride, 1, (long long)a.nf * a.S * a.ldv, a.err, 18) = r;
-    }
-}
-
-// MODE 1 (plain): the output is the transform alone (no window, base or previous-output terms,
-// column sums or time reversal, a_mdc = 1); MODE 0: the general epilogue; MODE 2: the general
-// epilogue with the LSQR x/w step of IrfftArgs fused in.  The inverse scale multiplies the
-// spectrum as it is loaded.  FUSE (aligned path, MODES 0 and 2): the epilogue also keeps its
-// outputs (windowed by fwd_cut) in the tile, and the kernel ends with their forward transform into
-// fwd_X -- the transform the next product of an LSQR iteration needs, without reading the output
-// back from memory.
-template <int N1, int N2, int MODE, int PP, bool FUSE = false>
-__global__ void __launch_bounds__(FFT_THREADS, MODE == 2 ? 2 : 3) irfft4_kernel(IrfftArgs a) {
-    constexpr bool PLAIN = MODE == 1, XW = MODE == 2;
-    static_assert(!(FUSE && PLAIN), "the fused forward transform follows the general epilogue");
-    using F = FourStep<N1, N2, PP>;
-    constexpr int NT = F::NT, CT = F::CT, P = F::P;
-    if (a.active && *a.active == 0) return;
-    extern __shared__ __align__(16) float2 sm2[];
-    float2* tw = sm2;
-    float2* z = sm2 + NT / 2;
-    // column-sum reduction: on the consumed tile, or (FUSE: the tile is transformed again) after it
-    double* red = reinterpret_cast<double*>(FUSE ? z + F::ZSIZE : z);
-    const int c0 = blockIdx.x * CT;
-    for (int i = threadIdx.x; i < NT / 2; i += FFT_THREADS) tw[i] = cconj(a.tw[i]);
-    // rows no bin of the slab [k0, k0 + nf) reaches are zero (16-byte stores, P is even)
-    const int kend = a.k0 + a.nf;
-    for (int idx = threadIdx.x; idx < NT * (P / 2); idx += FFT_THREADS) {
-        const int k = idx / (P / 2);
-        const bool hit = (k >= a.k0 && k < kend) || (NT - k >= a.k0 && NT - k < kend);
-        if (!hit) *reinterpret_cast<float4*>(z + F::zi(k, 2 * (idx % (P / 2)))) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const float isc = a.scale;
-    // Each loaded entry kk < nf (bin kb = k0 + kk) of the two columns fills Z[kb] and its
-    // Hermitian mirror Z[NT - kb].  Every thread keeps one column pair j (FFT_THREADS is a
-    // multiple of P), so its two spectrum columns are located once.
-    {
-        const int j = threadIdx.x % P, ca = c0 + 2 * j;
-        const size_t kstride = (size_t)a.S * a.ldv;
-        const float2* pa = nullptr;
-        const float2* pb = nullptr;
-        size_t paoff = 0, pboff = 0;
-        if (ca < a.C) {
-            const int sa = ca / a.nv, va = ca - sa * a.nv;
-            paoff = (size_t)sa * a.ldv + a.voff + va;
-            pa = a.Y + paoff;
-            if (ca + 1 < a.C) {
-                const int sb = (ca + 1) / a.nv, vb = ca + 1 - sb * a.nv;
-                pboff = (size_t)sb * a.ldv + a.voff + vb;
-                pb = a.Y + pboff;
-            }
-        }
-        // both columns as one 16-byte load when they are adjacent and every row keeps the alignment
-        const bool pair16 = pb == pa + 1 && ((uintptr_t)pa & 15) == 0 && (kstride & 1) == 0;
-        constexpr int B = 4, STEP = FFT_THREADS / P;
-#pragma unroll 1
-        for (int kk0 = threadIdx.x / P; kk0 < a.nf; kk0 += B * STEP) {
-            float2 A[B], Bv[B];
-#pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int kk = kk0 + u * STEP;
-                A[u] = make_float2(0.f, 0.f);
-                Bv[u] = A[u];
-                if (kk < a.nf && pa) {
-                    const size_t o = (size_t)kk * kstride;
-                    if (pair16) {
-                        const float4 q = *reinterpret_cast<const float4*>(MDC_AT(a.Y, paoff + o, 2, (long long)a.nf * a.S * a.ldv, a.err, 20));
-                        A[u] = make_float2(q.x, q.y);
-                        Bv[u] = make_float2(q.z, q.w);
-                    } else {
-                        A[u] = *MDC_AT(a.Y, paoff + o, 1, (long long)a.nf * a.S * a.ldv, a.err, 21);
-                        if (pb) Bv[u] = *MDC_AT(a.Y, pboff + o, 1, (long long)a.nf * a.S * a.ldv, a.err, 22);
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int kk = kk0 + u * STEP;
-                if (kk >= a.nf) continue;
-                const int kb = kk + a.k0;
-                float2 Av = make_float2(isc * A[u].x, isc * A[u].y), Bw = make_float2(isc * Bv[u].x, isc * Bv[u].y);
-                if (a.conj_in) { Av.y = -Av.y; Bw.y = -Bw.y; }
-                if (kb == 0 || 2 * kb == NT) { Av.y = 0.f; Bw.y = 0.f; }
-                z[F::zi(kb, j)] = make_float2(Av.x - Bw.y, Av.y + Bw.x);
-                if (kb > 0 && 2 * kb < NT) z[F::zi(NT - kb, j)] = make_float2(Av.x + Bw.y, Bw.x - Av.y);
-            }
-        }
-    }
-    __syncthreads();
-    four_step<N1, N2, true, false, PP>(z, tw);
-
-    if constexpr (PLAIN) {
-        // storage row rho holds time sample t = (rho % N2) * N1 + rho / N2
-        if (a.vec4) {
-            constexpr int Q = CT / 4, TS = FFT_THREADS / Q;
-            const int q = threadIdx.x % Q, cq = c0 + 4 * q;
-            if (cq < a.C) {
-#pragma unroll 4
-                for (int rho = threadIdx.x / Q; rho < NT; rho += TS) {
-                    const int t = (rho % N2) * N1 + rho / N2;
-                    *reinterpret_cast<float4*>(MDC_AT(a.out, (size_t)t * a.C + cq, 4, (long long)NT * a.C, a.err, 23)) =
-                        *reinterpret_cast<const float4*>(z + F::zi(rho, 2 * q));
-                }
-            }
-        } else {
-            const int cl = threadIdx.x % CT, c = c0 + cl;
-            if (c < a.C) {
-                for (int rho = threadIdx.x / CT; rho < NT; rho += FFT_THREADS / CT) {
-                    const int t = (rho % N2) * N1 + rho / N2;
-                    const float2 zz = z[F::zi(rho, cl >> 1)];
-                    *MDC_AT(a.out, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 24) = (cl & 1) ? zz.y : zz.x;
-                }
-            }
-        }
-        return;
-    }
-    const float am = coef(a.a_mdc), ab = coef(a.a_base), ap = coef(a.a_prev);
-    const bool has_prev = (a.a_prev.h != 0.f) || (a.a_prev.d != nullptr);
-    float xkx = 0.f, xkw = 0.f, xia = 0.f;
-    if constexpr (XW) {
-        xkx = (float)*a.xw_kx;
-        xkw = (float)*a.xw_kw;
-        xia = (float)*a.xw_ia;
-    }
-    if (a.vec4) {
-        // four adjacent columns per thread: 16-byte loads and stores
-        constexpr int Q = CT / 4, TS = FFT_THREADS / Q, PER = NT / TS, BB = XW ? 2 : 4, B = PER < BB ? PER : BB;
-        const int q = threadIdx.x % Q, t0 = threadIdx.x / Q, cq = c0 + 4 * q;
-        const bool want_ss = a.colsum != nullptr;
-        float ss[4] = {0.f, 0.f, 0.f, 0.f};   // per-thread partial sums of squares (<= 16 terms)
-        if (cq < a.C) {
-            int cut[4], fcut[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                cut[i] = a.cut ? *MDC_AT(a.cut, cq + i, 1, a.C, a.err, 25) : 0x7fffffff;
-                fcut[i] = (FUSE && a.fwd_cut) ? *MDC_AT(a.fwd_cut, cq + i, 1, a.C, a.err, 26) : 0x7fffffff;
-            }
-#pragma unroll 1
-            for (int b0 = 0; b0 < PER; b0 += B) {
-                // storage row rho holds time sample t = (rho % N2) * N1 + rho / N2
-                float4 bv[B], pv[B], wv[XW ? B : 1], xv[XW ? B : 1];
-#pragma unroll
-                for (int u = 0; u < B; ++u) {
-                    const int rho = t0 + (b0 + u) * TS;
-                    const size_t o = (size_t)((rho % N2) * N1 + rho / N2) * a.C + cq;
-                    bv[u] = a.base ? *reinterpret_cast<const float4*>(MDC_AT(a.base, o, 4, (long long)NT * a.C, a.err, 27))
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-                    pv[u] = has_prev ? *reinterpret_cast<const float4*>(MDC_AT(a.out, o, 4, (long long)NT * a.C, a.err, 28))
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-                    if constexpr (XW) {
-                        wv[u] = *reinterpret_cast<const float4*>(MDC_AT(a.xw_w, o, 4, (long long)NT * a.C, a.err, 29));
-                        xv[u] = *reinterpret_cast<const float4*>(MDC_AT(a.xw_x, o, 4, (long long)NT * a.C, a.err, 30));
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < B; ++u) {
-                    const int rho = t0 + (b0 + u) * TS;
-                    const int t = (rho % N2) * N1 + rho / N2;
-                    const float4 zz = *reinterpret_cast<const float4*>(z + F::zi(rho, 2 * q));
-                    const float2 z0 = make_float2(zz.x, zz.y), z1 = make_float2(zz.z, zz.w);
-                    const int tau = t < (NT >> 1) ? t : NT - t;
-                    float v[4] = {z0.x, z0.y, z1.x, z1.y};
-                    const float bb[4] = {bv[u].x, bv[u].y, bv[u].z, bv[u].w};
-                    const float pp[4] = {pv[u].x, pv[u].y, pv[u].z, pv[u].w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float val = tau >= cut[i] ? 0.f : v[i];          // scale applied at load
-                        v[i] = am * val + ab * bb[i] + ap * pp[i];
-                        if (want_ss) ss[i] = fmaf(v[i], v[i], ss[i]);
-                    }
-                    const size_t o = (size_t)t * a.C + cq;
-                    *reinterpret_cast<float4*>(MDC_AT(a.out, o, 4, (long long)NT * a.C, a.err, 31)) = make_float4(v[0], v[1], v[2], v[3]);
-                    if constexpr (FUSE) {
-                        // the same tile slot, windowed for the forward transform
-                        *reinterpret_cast<float4*>(z + F::zi(rho, 2 * q)) =
-                            make_float4(tau >= fcut[0] ? 0.f : v[0], tau >= fcut[1] ? 0.f : v[1],
-                                        tau >= fcut[2] ? 0.f : v[2], tau >= fcut[3] ? 0.f : v[3]);
-                    }
-                    if constexpr (XW) {
-                        const float ww[4] = {wv[u].x, wv[u].y, wv[u].z, wv[u].w};
-                        const float xx[4] = {xv[u].x, xv[u].y, xv[u].z, xv[u].w};
-                        float nw[4], nx[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            nx[i] = fmaf(xkx, ww[i], xx[i]);
-                            nw[i] = fmaf(xkw, ww[i], xia * pp[i]);
-                        }
-                        *reinterpret_cast<float4*>(MDC_AT(a.xw_x, o, 4, (long long)NT * a.C, a.err, 32)) = make_float4(nx[0], nx[1], nx[2], nx[3]);
-                        *reinterpret_cast<float4*>(MDC_AT(a.xw_w, o, 4, (long long)NT * a.C, a.err, 33)) = make_float4(nw[0], nw[1], nw[2], nw[3]);
-                    }
-                }
-            }
-        }
-        if (a.colsum) {
-            __syncthreads();                             // every thread is done reading the tile
-#pragma unroll
-            for (int i = 0; i < 4; ++i) red[4 * threadIdx.x + i] = (double)ss[i];
-            __syncthreads();
-            if (threadIdx.x < CT && c0 + (int)threadIdx.x < a.C) {
-                const int qq = threadIdx.x / 4, ii = threadIdx.x % 4;
-                double tot = 0.0;
-                for (int tt = qq; tt < FFT_THREADS; tt += Q) tot += red[4 * tt + ii];
-                *MDC_AT(a.colsum, c0 + threadIdx.x, 1, a.C, a.err, 34) = tot;
-            }
-        }
-        if constexpr (FUSE) {
-            __syncthreads();                             // every output is in the tile
-            fused_forward<N1, N2, PP>(a, z, tw, c0);
-        }
-        return;
-    }
-    const int cl = threadIdx.x % CT, c = c0 + cl;
-    const bool want_ss = a.colsum != nullptr;
-    float ss = 0.f;   // per-thread partial sum of squares (<= 64 terms)
-    if (c < a.C) {
-        const int cut = a.cut ? *MDC_AT(a.cut, c, 1, a.C, a.err, 35) : 0x7fffffff;
-        constexpr int TS = FFT_THREADS / CT, PER = NT / TS, B = PER < 8 ? PER : 8;
-        const int t0 = threadIdx.x / CT;
-#pragma unroll 1
-        for (int b0 = 0; b0 < PER; b0 += B) {
-            float bv[B], pv[B], wv[XW ? B : 1], xv[XW ? B : 1];
-#pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int rho = t0 + (b0 + u) * TS;
-                const int t = (rho % N2) * N1 + rho / N2;
-                const int to = a.reverse_out ? ((NT - t) & (NT - 1)) : t;
-                bv[u] = a.base ? *MDC_AT(a.base, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 36) : 0.f;
-                pv[u] = has_prev ? *MDC_AT(a.out, (size_t)to * a.C + c, 1, (long long)NT * a.C, a.err, 37) : 0.f;
-                if constexpr (XW) {
-                    wv[u] = *MDC_AT(a.xw_w, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 38);
-                    xv[u] = *MDC_AT(a.xw_x, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 39);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < B; ++u) {
-                const int rho = t0 + (b0 + u) * TS;
-                const int t = (rho % N2) * N1 + rho / N2;
-                const float2 zz = z[F::zi(rho, cl >> 1)];
-                float val = (cl & 1) ? zz.y : zz.x;                      // scale applied at load
-                const int tau = t < (NT >> 1) ? t : NT - t;
-                if (tau >= cut) val = 0.f;
-                const float r = am * val + ab * bv[u] + ap * pv[u];
-                const int to = a.reverse_out ? ((NT - t) & (NT - 1)) : t;
-                *MDC_AT(a.out, (size_t)to * a.C + c, 1, (long long)NT * a.C, a.err, 40) = r;
-                if (want_ss) ss = fmaf(r, r, ss);
-                if constexpr (XW) {
-                    *MDC_AT(a.xw_x, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 41) = fmaf(xkx, wv[u], xv[u]);
-                    *MDC_AT(a.xw_w, (size_t)t * a.C + c, 1, (long long)NT * a.C, a.err, 42) = fmaf(xkw, wv[u], xia * pv[u]);
-                }
-            }
-        }
-    }
-    if (a.colsum) {
-        __syncthreads();                                 // every thread is done reading the tile
-        red[threadIdx.x] = (double)ss;
-        __syncthreads();
-        if (threadIdx.x < CT && c < a.C) {
-            double tot = 0.0;
-            for (int i = threadIdx.x; i < FFT_THREADS; i += CT) tot += red[i];
-            *MDC_AT(a.colsum, c, 1, a.C, a.err, 10) = tot;
         }
     }
 }
@@ -1016,7 +489,7 @@ __global__ void __launch_bounds__(FFT_THREADS, PLAIN ? 3 : 2) irfft_half_kernel(
         }
     }
     __syncthreads();
-    four_step<N1, N2, true, true>(z, twc);
+    four_step<N1, N2, true>(z, twc);
 
     // Row rho holds complex sample n = (rho % N2) * N1 + rho / N2, i.e. real samples 2n (real
     // part) and 2n + 1 (imaginary part).
@@ -1183,12 +656,6 @@ __global__ void __launch_bounds__(FFT_THREADS, PLAIN ? 3 : 2) irfft_half_kernel(
     }
 }
 
-// The transform alone: no window, base or previous-output terms, column sums or reversal.
-inline bool irfft_plain(const IrfftArgs& a) {
-    return !a.cut && !a.base && !a.colsum && !a.reverse_out && a.a_mdc.h == 1.f && !a.a_mdc.d &&
-           a.a_prev.h == 0.f && !a.a_prev.d && !a.xw_w && !a.fwd_X;
-}
-
 template <int N1, int N2, bool WIN, bool X2>
 void rfft_half_go(mdc_plan* p, const RfftArgs& a, cudaStream_t s) {
     using H = HalfStep<N1, N2>;
@@ -1242,17 +709,10 @@ void rfft4_go(mdc_plan* p, const RfftArgs& a, cudaStream_t s) {
     rfft4_kernel<N1, N2, WIN, X2, PP><<<(a.C + F::CT - 1) / F::CT, FFT_THREADS, F::smem_full, s>>>(a);
 }
 
-// Few columns: the default tile would leave most SMs idle (fewer CTAs than half the SMs); smaller
-// tiles then shorten each CTA's work.  (With one or more default CTAs per SM the smaller tiles only
-// add waves: measured slower at 3721 columns of 1024 samples.)
-template <int N1, int N2>
-constexpr int few_cols_p() { return 1024 / (N1 * N2) > 2 ? 1024 / (N1 * N2) : 2; }
-inline bool few_columns(int C, int ct) { return (C + ct - 1) / ct < 148 / 2; }
-
 template <int N1, int N2>
 void rfft4_launch(mdc_plan* p, const RfftArgs& a0, cudaStream_t s) {
     RfftArgs a = a0;
-    a.vec4 = (a.C % 4 == 0) && ((uintptr_t)a.x % 16 == 0) && (!a.x2 || (uintptr_t)a.x2 % 16 == 0);
+    a.v2 = (a.C % 2 == 0) && ((uintptr_t)a.x % 8 == 0) && ((uintptr_t)a.x2 % 8 == 0);
     constexpr int PS = few_cols_p<N1, N2>();
     const bool few = few_columns(a.C, FourStep<N1, N2>::CT) && PS < FourStep<N1, N2>::P;
     if (a.cut) {
@@ -1265,40 +725,6 @@ void rfft4_launch(mdc_plan* p, const RfftArgs& a0, cudaStream_t s) {
     } else {
         rfft4_go<N1, N2, false, false, 0>(p, a, s);
     }
-}
-
-template <int N1, int N2, int MODE, int PP, bool FUSE = false>
-void irfft4_go(mdc_plan* p, const IrfftArgs& a, cudaStream_t s) {
-    using F = FourStep<N1, N2, PP>;
-    // FUSE: the column-sum reduction buffer follows the tile
-    constexpr size_t smem = F::smem + (FUSE ? (size_t)FFT_THREADS * 4 * sizeof(double) : 0);
-    static SmemLimit attr;
-    attr.ensure(irfft4_kernel<N1, N2, MODE, PP, FUSE>, (int)smem);
-    LaunchScope ls(p, s, MDC_KC_IRFFT);
-    irfft4_kernel<N1, N2, MODE, PP, FUSE><<<(a.C + F::CT - 1) / F::CT, FFT_THREADS, smem, s>>>(a);
-}
-
-// Returns true if the kernel also made the forward transform of IrfftArgs::fwd_X.
-template <int N1, int N2>
-bool irfft4_launch(mdc_plan* p, const IrfftArgs& a0, cudaStream_t s) {
-    IrfftArgs a = a0;
-    a.vec4 = (a.C % 4 == 0) && !a.reverse_out && ((uintptr_t)a.out % 16 == 0) &&
-             (!a.base || (uintptr_t)a.base % 16 == 0) &&
-             (!a.xw_w || ((uintptr_t)a.xw_w % 16 == 0 && (uintptr_t)a.xw_x % 16 == 0));
-    constexpr int PS = few_cols_p<N1, N2>();
-    const bool few = few_columns(a.C, FourStep<N1, N2>::CT) && PS < FourStep<N1, N2>::P;
-    const bool fuse = a.fwd_X && a.vec4 && !a.reverse_out;
-    if (irfft_plain(a)) {
-        if (few) irfft4_go<N1, N2, 1, PS>(p, a, s);
-        else irfft4_go<N1, N2, 1, 0>(p, a, s);
-    } else if (a.xw_w) {
-        if (fuse) irfft4_go<N1, N2, 2, 0, true>(p, a, s);
-        else irfft4_go<N1, N2, 2, 0>(p, a, s);
-    } else {
-        if (fuse) irfft4_go<N1, N2, 0, 0, true>(p, a, s);
-        else irfft4_go<N1, N2, 0, 0>(p, a, s);
-    }
-    return fuse;
 }
 
 int tile_log_columns(int nt) {
