@@ -100,73 +100,7 @@ __device__ __forceinline__ void cfma_conj(float2& acc, float2 a, float2 b) {
 __device__ __forceinline__ float4 ld_stream(const float4* p) { return __ldcs(p); }
 
 // ---- complex64 GEMV kernels (begin)
-// complex64 specialisations: one warp per row, X(w) interleaved in shared memory (C64 keeps
-// two complex values per vector, so lanes already read distinct words).
-template <int NVC>
-__global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_c64(
-    const float4* __restrict__ G, int ldg, int nr, int ns,
-    const float2* __restrict__ X, int ldi, int voff_i,
-    float2* __restrict__ Y, int ldo, int voff_o, const int* active, int* err) {
-    if (active && *active == 0) return;
-    extern __shared__ __align__(16) float2 xs[];   // [ldg][NVC]
-    const int k = blockIdx.y;
-    const float2* Xk = X + (size_t)k * ns * ldi + voff_i;
-    for (int i = threadIdx.x; i < ldg * NVC; i += GEMV_THREADS) {
-        const int s = i / NVC, v = i - s * NVC;
-        xs[i] = s < ns && MDC_INB((size_t)k * ns * ldi + voff_i + (size_t)s * ldi + v, 1, (long long)gridDim.y * ns * ldi, err, 100)
-                    ? Xk[(size_t)s * ldi + v] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nvec = ldg >> 1;
-    const int r0 = blockIdx.x * FWD_ROWS_PER_CTA;
-    const int r1 = min(r0 + FWD_ROWS_PER_CTA, nr);
-    for (int r = r0 + warp; r < r1; r += GEMV_THREADS / 32) {
-        if (!MDC_INB(((size_t)k * nr + r) * nvec, nvec, (long long)gridDim.y * nr * nvec, err, 101)) continue;
-        const float4* g = G + ((size_t)k * nr + r) * nvec;
-        float2 acc[NVC];
-#pragma unroll
-        for (int v = 0; v < NVC; ++v) acc[v] = make_float2(0.f, 0.f);
-        int i = lane;
-        for (; i + 96 < nvec; i += 128) {
-            float4 gv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) gv[u] = ld_stream(g + i + 32 * u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int s = 2 * (i + 32 * u);
-#pragma unroll
-                for (int v = 0; v < NVC; ++v) {
-                    cfma(acc[v], make_float2(gv[u].x, gv[u].y), xs[s * NVC + v]);
-                    cfma(acc[v], make_float2(gv[u].z, gv[u].w), xs[(s + 1) * NVC + v]);
-                }
-            }
-        }
-        for (; i < nvec; i += 32) {
-            const float4 gv = ld_stream(g + i);
-            const int s = 2 * i;
-#pragma unroll
-            for (int v = 0; v < NVC; ++v) {
-                cfma(acc[v], make_float2(gv.x, gv.y), xs[s * NVC + v]);
-                cfma(acc[v], make_float2(gv.z, gv.w), xs[(s + 1) * NVC + v]);
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < NVC; ++v) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                acc[v].x += __shfl_xor_sync(0xffffffffu, acc[v].x, off);
-                acc[v].y += __shfl_xor_sync(0xffffffffu, acc[v].y, off);
-            }
-        }
-        if (lane == 0 && MDC_INB(((size_t)k * nr + r) * ldo + voff_o, NVC, (long long)gridDim.y * nr * ldo, err, 102)) {
-            float2* y = Y + ((size_t)k * nr + r) * ldo + voff_o;
-#pragma unroll
-            for (int v = 0; v < NVC; ++v) y[v] = acc[v];
-        }
-    }
-}
-
+// complex64 specialisation of the adjoint
 constexpr int ADJ_TILE = 64;   // complex columns per CTA (one 512-byte row segment)
 
 template <int NVC>
@@ -239,76 +173,136 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_adj_c64(
     }
 }
 
-// ---- complex64 GEMV kernels (end)
 
-// Forward GEMV.  X(w) is staged de-interleaved by vector lane position:
-// xs[(j * nvec + i) * NVC + v] = X[CPV * i + j][v], so the 32 lanes of a warp, which
-// hold vectors i..i+31, read consecutive shared-memory words for every j.
+// X(w) is staged de-interleaved by vector lane position, one plane per column and position:
+// xs[(v * CPV + j) * pitch + i] = X[CPV * i + j][v], so the 32 lanes of a warp, which hold vectors
+// i..i+31, read consecutive shared-memory words for every j and v.
+//
+// A warp walks RB rows at once: RB * U vectors of G in flight per lane, and every X value read from
+// shared memory serves RB rows.  (One row at a time, short rows exposed a memory latency per vector, and
+// four interleaved columns read shared memory eight ways conflicted.)  Bound by HBM on long rows.
+// Complex64, before / now: 1 column on 441^2 x 64 28.9 / 24.5 us; 4 columns on 441^2 x 64 58 / 26 us,
+// 1681^2 x 150 903 / 591 us, 3721^2 x 60 1691 / 1121 us (adjoint 1005 us); 3 columns there 1478 / 1000
+// us; float16, 1 and 4 columns on 3721^2 x 60 583 / 503 and 1667 / 1025 us.  Every lane adds its
+// products in ascending order of the vectors, whatever RB and U.
+// RB and U by measurement on 441^2, 1681^2, 3721 x 841 and 3721^2 kernels.  SHAPE: whole rows of X staged,
+// chunks of it, or whole rows of more than LONG_ROW columns, where one column of complex64 and split
+// FP16 streams best one row at a time (3721^2 x 200: 3.13 ms, two rows at once 3.17 ms; 441^2 x 64: 29
+// us, 25 us).
+enum { ROWS_WHOLE = 0, ROWS_CHUNK = 1, ROWS_LONG = 2 };
+constexpr int LONG_ROW = 2048;
+template <int FMT, int NVC, int SHAPE> struct FwdRows {
+    static constexpr bool H16 = FMT == MDC_C16F || FMT == MDC_CBF16, WIDE4 = SHAPE == ROWS_CHUNK && NVC == 4;
+    static constexpr int RB = SHAPE == ROWS_LONG ? 1
+                              : (H16 && NVC == 1) || ((H16 || FMT == MDC_C64) && WIDE4) ? 4 : 2;      // rows at once
+    static constexpr int U = SHAPE == ROWS_LONG ? 4
+                             : FMT == MDC_C64 ? (WIDE4 ? 1 : 2) : (H16 && NVC > 1) || (FMT == MDC_C32S && NVC == 2) ? 2 : 1;
+};
+
+// Place of X[CPV * i + j][v] in shared memory: planes (see above), or, for one column of complex64,
+// both values of a vector side by side (one 16-byte read).
 template <int FMT, int NVC>
+__device__ __forceinline__ int xs_at(int v, int j, int i, int pitch) {
+    return FMT == MDC_C64 && NVC == 1 ? 2 * i + j : (v * Fmt<FMT>::CPV + j) * pitch + i;
+}
+
+// acc[q][v] += sum over vectors i = i0 + lane, + 32, ... < i1 of row g[q] times X.
+template <int FMT, int NVC, int RB, int U>
+__device__ __forceinline__ void gemv_rows(const uint4* const (&g)[RB], int i0, int i1, int64_t lo, const float2* xs,
+                                          int pitch, int xbase, float2 (&acc)[RB][NVC]) {
+    constexpr int CPV = Fmt<FMT>::CPV;
+    auto apply = [&](const float2 (&c)[RB][CPV], int i) {
+#pragma unroll
+        for (int j = 0; j < CPV; ++j)
+#pragma unroll
+            for (int v = 0; v < NVC; ++v) {
+                const float2 x = xs[xs_at<FMT, NVC>(v, j, i - xbase, pitch)];
+#pragma unroll
+                for (int q = 0; q < RB; ++q) cfma(acc[q][v], c[q][j], x);
+            }
+    };
+    int i = i0 + (threadIdx.x & 31);
+    for (; i + 32 * (U - 1) < i1; i += 32 * U) {
+        float2 c[U][RB][CPV];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < RB; ++q) load_decode<FMT>(g[q], i + 32 * u, lo, c[u][q]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) apply(c[u], i + 32 * u);
+    }
+    for (; i < i1; i += 32) {
+        float2 c[RB][CPV];
+#pragma unroll
+        for (int q = 0; q < RB; ++q) load_decode<FMT>(g[q], i, lo, c[q]);
+        apply(c, i);
+    }
+}
+
+// Sum over the warp's lanes, row scale, store (rows r[q] < nr only).
+template <int FMT, int NVC, int RB>
+__device__ __forceinline__ void gemv_rows_store(float2 (&acc)[RB][NVC], const int (&r)[RB], int nr,
+                                                const float* __restrict__ gscale, float2* __restrict__ Y, int ldo,
+                                                int voff_o, int* err) {
+    const int k = blockIdx.y;
+#pragma unroll
+    for (int q = 0; q < RB; ++q) {
+#pragma unroll
+        for (int v = 0; v < NVC; ++v)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                acc[q][v].x += __shfl_xor_sync(0xffffffffu, acc[q][v].x, off);
+                acc[q][v].y += __shfl_xor_sync(0xffffffffu, acc[q][v].y, off);
+            }
+        if ((threadIdx.x & 31) == 0 && r[q] < nr &&
+            MDC_INB(((size_t)k * nr + r[q]) * ldo + voff_o, NVC, (long long)gridDim.y * nr * ldo, err, 109)) {
+            const float sc = (FMT == MDC_C64) ? 1.f : gscale[(size_t)k * nr + r[q]];
+            float2* y = Y + ((size_t)k * nr + r[q]) * ldo + voff_o;
+#pragma unroll
+            for (int v = 0; v < NVC; ++v) y[v] = make_float2(acc[q][v].x * sc, acc[q][v].y * sc);
+        }
+    }
+}
+
+template <int FMT, int NVC, int SHAPE>
 __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd(
     const uint4* __restrict__ G, int ldg, int nr, int ns, const float* __restrict__ gscale,
     const float2* __restrict__ X, int ldi, int voff_i,
     float2* __restrict__ Y, int ldo, int voff_o, const int* active, int64_t lo, int* err) {
-    constexpr int CPV = Fmt<FMT>::CPV;
+    using FR = FwdRows<FMT, NVC, SHAPE>;
+    constexpr int CPV = Fmt<FMT>::CPV, RB = FR::RB, W = GEMV_THREADS / 32;
     if (active && *active == 0) return;
-    extern __shared__ __align__(16) float2 xs[];
+    extern __shared__ __align__(16) float2 xs[];   // [NVC][CPV][nvec]
     const int k = blockIdx.y;
     const int nvec = ldg / CPV;
     const float2* Xk = X + (size_t)k * ns * ldi + voff_i;
     for (int e = threadIdx.x; e < ldg * NVC; e += GEMV_THREADS) {
         const int s = e / NVC, v = e - s * NVC;
         const int i = s / CPV, j = s - i * CPV;
-        xs[(j * nvec + i) * NVC + v] =
+        xs[xs_at<FMT, NVC>(v, j, i, nvec)] =
             s < ns && MDC_INB((size_t)k * ns * ldi + voff_i + (size_t)s * ldi + v, 1, (long long)gridDim.y * ns * ldi, err, 106)
                 ? Xk[(size_t)s * ldi + v] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = blockIdx.x * FWD_ROWS_PER_CTA;
-    const int r1 = min(r0 + FWD_ROWS_PER_CTA, nr);
-    for (int r = r0 + warp; r < r1; r += GEMV_THREADS / 32) {
-        if (!MDC_INB(((size_t)k * nr + r) * nvec, nvec, (long long)gridDim.y * nr * nvec, err, 107)) continue;
-        const uint4* g = G + ((size_t)k * nr + r) * nvec;
-        float2 acc[NVC];
+    const int r1 = min((int)(blockIdx.x + 1) * FWD_ROWS_PER_CTA, nr);
+    for (int r0 = blockIdx.x * FWD_ROWS_PER_CTA + (threadIdx.x >> 5); r0 < r1; r0 += W * RB) {
+        int r[RB];
+        const uint4* g[RB];
+        float2 acc[RB][NVC];
 #pragma unroll
-        for (int v = 0; v < NVC; ++v) acc[v] = make_float2(0.f, 0.f);
-        int i = lane;
-        for (; i + 96 < nvec; i += 128) {
-            float2 c4[4][CPV];
+        for (int q = 0; q < RB; ++q) {
+            r[q] = r0 + W * q;
+            const int rc = min(r[q], nr - 1);              // past the end: a row that exists, not stored
+            g[q] = G + (MDC_INB(((size_t)k * nr + rc) * nvec, nvec, (long long)gridDim.y * nr * nvec, err, 107)
+                            ? ((size_t)k * nr + rc) * nvec : 0);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) load_decode<FMT>(g, i + 32 * u, lo, c4[u]);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-#pragma unroll
-                for (int j = 0; j < CPV; ++j)
-#pragma unroll
-                    for (int v = 0; v < NVC; ++v) cfma(acc[v], c4[u][j], xs[(j * nvec + i + 32 * u) * NVC + v]);
-            }
+            for (int v = 0; v < NVC; ++v) acc[q][v] = make_float2(0.f, 0.f);
         }
-        for (; i < nvec; i += 32) {
-            float2 c[CPV];
-            load_decode<FMT>(g, i, lo, c);
-#pragma unroll
-            for (int j = 0; j < CPV; ++j)
-#pragma unroll
-                for (int v = 0; v < NVC; ++v) cfma(acc[v], c[j], xs[(j * nvec + i) * NVC + v]);
-        }
-#pragma unroll
-        for (int v = 0; v < NVC; ++v) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                acc[v].x += __shfl_xor_sync(0xffffffffu, acc[v].x, off);
-                acc[v].y += __shfl_xor_sync(0xffffffffu, acc[v].y, off);
-            }
-        }
-        if (lane == 0 && MDC_INB(((size_t)k * nr + r) * ldo + voff_o, NVC, (long long)gridDim.y * nr * ldo, err, 109)) {
-            const float sc = (FMT == MDC_C64) ? 1.f : gscale[(size_t)k * nr + r];
-            float2* y = Y + ((size_t)k * nr + r) * ldo + voff_o;
-#pragma unroll
-            for (int v = 0; v < NVC; ++v) y[v] = make_float2(acc[v].x * sc, acc[v].y * sc);
-        }
+        gemv_rows<FMT, NVC, RB, FR::U>(g, 0, nvec, lo, xs, nvec, 0, acc);
+        gemv_rows_store<FMT, NVC, RB>(acc, r, nr, gscale, Y, ldo, voff_o, err);
     }
 }
+// ---- complex64 GEMV kernels (end)
 
 // Adjoint GEMV: a CTA owns TILE = 32 * CPV adjacent columns s of one frequency (one 512-byte
 // segment of every row); warp w walks rows r = w, w + 8, ...; the row scale is folded into Y.
@@ -417,29 +411,38 @@ struct AdjChunk {
     static constexpr int CHR = ((GEMV_CHUNK_BYTES / (8 * NVC)) / 32) * 32;
 };
 
-// Forward: the CTA's 32 rows, warp w owning rows r0 + w + 8 q (q < 4) with their partial sums
-// held in registers across chunks.
+// Forward: the CTA's 32 rows, warp w owning rows r0 + w + 8 q (q < 4) with their partial sums held in
+// registers across chunks.
 template <int FMT, int NVC>
 __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_chunked(
     const uint4* __restrict__ G, int ldg, int nr, int ns, const float* __restrict__ gscale,
     const float2* __restrict__ X, int ldi, int voff_i,
     float2* __restrict__ Y, int ldo, int voff_o, const int* active, int64_t lo, int* err) {
-    constexpr int CPV = Fmt<FMT>::CPV;
+    using FR = FwdRows<FMT, NVC, ROWS_CHUNK>;
+    constexpr int CPV = Fmt<FMT>::CPV, RB = FR::RB;
     constexpr int CHV = FwdChunk<FMT, NVC>::CHV;
     constexpr int W = GEMV_THREADS / 32;
-    constexpr int RPW = FWD_CHUNK_ROWS / W;
+    constexpr int NB = FWD_CHUNK_ROWS / (W * RB);      // batches of RB rows per warp
     if (active && *active == 0) return;
-    extern __shared__ __align__(16) float2 xs[];   // [CPV][CHV][NVC]
+    extern __shared__ __align__(16) float2 xs[];   // [NVC][CPV][CHV]
     const int k = blockIdx.y;
     const int nvec = ldg / CPV;
     const float2* Xk = X + (size_t)k * ns * ldi + voff_i;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rw = blockIdx.x * FWD_CHUNK_ROWS + warp;
-    float2 acc[RPW][NVC];
+    const int rw = blockIdx.x * FWD_CHUNK_ROWS + (threadIdx.x >> 5);
+    int r[NB][RB];
+    const uint4* g[NB][RB];
+    float2 acc[NB][RB][NVC];
 #pragma unroll
-    for (int q = 0; q < RPW; ++q)
+    for (int b = 0; b < NB; ++b)
 #pragma unroll
-        for (int v = 0; v < NVC; ++v) acc[q][v] = make_float2(0.f, 0.f);
+        for (int q = 0; q < RB; ++q) {
+            r[b][q] = rw + W * (b * RB + q);
+            const int rc = min(r[b][q], nr - 1);           // past the end: a row that exists, not stored
+            g[b][q] = G + (MDC_INB(((size_t)k * nr + rc) * nvec, nvec, (long long)gridDim.y * nr * nvec, err, 115)
+                               ? ((size_t)k * nr + rc) * nvec : 0);
+#pragma unroll
+            for (int v = 0; v < NVC; ++v) acc[b][q][v] = make_float2(0.f, 0.f);
+        }
     for (int c0 = 0; c0 < nvec; c0 += CHV) {
         const int c1 = min(c0 + CHV, nvec);
         __syncthreads();                               // the previous chunk has been consumed
@@ -447,60 +450,18 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_chunked(
             const int sl = e / NVC, v = e - sl * NVC;
             const int i = sl / CPV, j = sl - i * CPV;
             const int s = c0 * CPV + sl;
-            xs[(j * CHV + i) * NVC + v] =
+            xs[xs_at<FMT, NVC>(v, j, i, CHV)] =
                 s < ns && MDC_INB((size_t)k * ns * ldi + voff_i + (size_t)s * ldi + v, 1, (long long)gridDim.y * ns * ldi, err, 114)
                     ? Xk[(size_t)s * ldi + v] : make_float2(0.f, 0.f);
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < RPW; ++q) {
-            const int r = rw + W * q;
-            if (r >= nr) break;                        // warp-uniform
-            if (!MDC_INB(((size_t)k * nr + r) * nvec, nvec, (long long)gridDim.y * nr * nvec, err, 115)) continue;
-            const uint4* g = G + ((size_t)k * nr + r) * nvec;
-            int i = c0 + lane;
-            for (; i + 96 < c1; i += 128) {
-                float2 c4[4][CPV];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) load_decode<FMT>(g, i + 32 * u, lo, c4[u]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-#pragma unroll
-                    for (int j = 0; j < CPV; ++j)
-#pragma unroll
-                        for (int v = 0; v < NVC; ++v)
-                            cfma(acc[q][v], c4[u][j], xs[(j * CHV + i - c0 + 32 * u) * NVC + v]);
-                }
-            }
-            for (; i < c1; i += 32) {
-                float2 c[CPV];
-                load_decode<FMT>(g, i, lo, c);
-#pragma unroll
-                for (int j = 0; j < CPV; ++j)
-#pragma unroll
-                    for (int v = 0; v < NVC; ++v) cfma(acc[q][v], c[j], xs[(j * CHV + i - c0) * NVC + v]);
-            }
-        }
+        for (int b = 0; b < NB; ++b)
+            if (r[b][0] < nr) gemv_rows<FMT, NVC, RB, FR::U>(g[b], c0, c1, lo, xs, CHV, c0, acc[b]);       // warp-uniform
     }
 #pragma unroll
-    for (int q = 0; q < RPW; ++q) {
-        const int r = rw + W * q;
-        if (r >= nr) break;
-#pragma unroll
-        for (int v = 0; v < NVC; ++v) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                acc[q][v].x += __shfl_xor_sync(0xffffffffu, acc[q][v].x, off);
-                acc[q][v].y += __shfl_xor_sync(0xffffffffu, acc[q][v].y, off);
-            }
-        }
-        if (lane == 0 && MDC_INB(((size_t)k * nr + r) * ldo + voff_o, NVC, (long long)gridDim.y * nr * ldo, err, 117)) {
-            const float sc = (FMT == MDC_C64) ? 1.f : gscale[(size_t)k * nr + r];
-            float2* y = Y + ((size_t)k * nr + r) * ldo + voff_o;
-#pragma unroll
-            for (int v = 0; v < NVC; ++v) y[v] = make_float2(acc[q][v].x * sc, acc[q][v].y * sc);
-        }
-    }
+    for (int b = 0; b < NB; ++b)
+        if (r[b][0] < nr) gemv_rows_store<FMT, NVC, RB>(acc[b], r[b], nr, gscale, Y, ldo, voff_o, err);
 }
 
 // Adjoint: Y(w) (row scales folded in) staged CHR rows at a time; per-lane column sums persist
@@ -770,20 +731,21 @@ void gemv_fwd_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
             ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
         return;
     }
-    static SmemLimit attr;
-    attr.ensure(gemv_fwd<FMT, NVC>, 220 * 1024);
     dim3 grid((p->nr + FWD_ROWS_PER_CTA - 1) / FWD_ROWS_PER_CTA, p->nf);
-    if constexpr (FMT == MDC_C64) {
-        static SmemLimit attr64;
-        attr64.ensure(gemv_fwd_c64<NVC>, 220 * 1024);
-        gemv_fwd_c64<NVC><<<grid, GEMV_THREADS, smem, s>>>(
-            reinterpret_cast<const float4*>(p->G), (int)p->ldg, p->nr, p->ns, in, ldi, voff_i, out, ldo,
-            voff_o, active, p->err_flag);
-        return;
+    auto go = [&](auto kern, SmemLimit& attr) {
+        attr.ensure(kern, 220 * 1024);
+        kern<<<grid, GEMV_THREADS, smem, s>>>(reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale,
+                                              in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+    };
+    if constexpr ((FMT == MDC_C64 || FMT == MDC_C32S) && NVC == 1) {
+        if (p->ldg > LONG_ROW) {
+            static SmemLimit attr_long;
+            go(gemv_fwd<FMT, NVC, ROWS_LONG>, attr_long);
+            return;
+        }
     }
-    gemv_fwd<FMT, NVC><<<grid, GEMV_THREADS, smem, s>>>(
-        reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out,
-        ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+    static SmemLimit attr;
+    go(gemv_fwd<FMT, NVC, ROWS_WHOLE>, attr);
 }
 
 template <int FMT, int NVC>
