@@ -143,8 +143,8 @@ struct Solver {
         cudaMemsetAsync(csU + C, 0, C * sizeof(double), s);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csU, 2 * C, part, nullptr);
-            norm_store<<<1, RED_THREADS, 0, s>>>(part, PART_CTAS, xs + X_DNORM);
+            const SumSource q = colsum_source(csU, 2 * C, part, nullptr, s);
+            norm_store<<<1, RED_THREADS, 0, s>>>(q.v, q.n, xs + X_DNORM);
         }
         if (D1()) {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
@@ -186,14 +186,14 @@ struct Solver {
         cudaMemsetAsync(sc, 0, S_COUNT * sizeof(double), s);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csU, 2 * C, part, nullptr);
-            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, resid0, act0 + 1);
+            const SumSource q = colsum_source(csU, 2 * C, part, nullptr, s);
+            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, resid0, act0 + 1);
         }
         apply_MH(act0 + 1, zero);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csV, 2 * C, part, act0 + 1);
-            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, act0 + 1);
+            const SumSource q = colsum_source(csV, 2 * C, part, act0 + 1, s);
+            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, act0 + 1);
         }
         LaunchScope ls(p, s, MDC_KC_SOLVER);
         if (zero_x) lsqr_xw_init<<<eg, 256, 0, s>>>(B, x1, x2, W1(), W2(), V1(), V2(), sc);
@@ -218,8 +218,8 @@ struct Solver {
         irfft(p, nv, 1, U2(), am, cut, V2(), CD(1.f, sc + S_INV_ALPHA), CD(1.f, sc + S_U_PREV), csU + C, 0, a,
               nullptr, nullptr, nv, cut, 1);
         LaunchScope ls(p, s, MDC_KC_SOLVER);
-        colsum_partials<<<PART_CTAS, 256, 0, s>>>(csU, 2 * C, part, a);
-        lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, a);
+        const SumSource q = colsum_source(csU, 2 * C, part, a, s);
+        lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a);
     }
     //   v-hat <- M^H u - beta v
     void iter_adj_pre(const int*) {}
@@ -234,8 +234,8 @@ struct Solver {
         irfft(p, 0, 0, V2(), CD(-1.f, sc + S_INV_BETA), nullptr, U2(), CD(1.f, sc + S_INV_BETA), vprev, csV + C, 0,
               a, x2, W2(), fuse_v ? 0 : -1, nullptr, 0);
         LaunchScope ls(p, s, MDC_KC_SOLVER);
-        colsum_partials<<<PART_CTAS, 256, 0, s>>>(csV, 2 * C, part, a);
-        lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, a, act0 + it + 1, resid0, itp, it,
+        const SumSource q = colsum_source(csV, 2 * C, part, a, s);
+        lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a, act0 + it + 1, resid0, itp, it,
                                                     niter, tol);
     }
     // The last rotation's pending x step (once per solve, after its last iteration).
@@ -339,8 +339,8 @@ void solve_body(Solver& S, const float* fd, int niter, int nref, int niter_ref, 
     if (want_final) {
         S.residual_pass(fm, fmp);
         LaunchScope ls(S.p, S.s, MDC_KC_SOLVER);
-        colsum_partials<<<PART_CTAS, 256, 0, S.s>>>(S.csU, 2 * S.C, S.part, nullptr);
-        norm_ratio<<<1, RED_THREADS, 0, S.s>>>(S.part, PART_CTAS, S.xs + X_DNORM, S.xs + X_FINAL);
+        const SumSource q = colsum_source(S.csU, 2 * S.C, S.part, nullptr, S.s);
+        norm_ratio<<<1, RED_THREADS, 0, S.s>>>(q.v, q.n, S.xs + X_DNORM, S.xs + X_FINAL);
     }
     if (gm || gp) S.greens(fd, fm, fmp, gm, gp);
 }
@@ -788,8 +788,8 @@ void finish_job(mdc_server* v, ServeJob* j) {
     S->residual_pass(j->x[0], j->x[1]);
     {
         LaunchScope ls(v->p, v->s, MDC_KC_SOLVER);
-        colsum_partials<<<PART_CTAS, 256, 0, v->s>>>(S->csU, 2 * S->C, S->part, nullptr);
-        norm_ratio<<<1, RED_THREADS, 0, v->s>>>(S->part, PART_CTAS, S->xs + X_DNORM, S->xs + X_FINAL);
+        const SumSource q = colsum_source(S->csU, 2 * S->C, S->part, nullptr, v->s);
+        norm_ratio<<<1, RED_THREADS, 0, v->s>>>(q.v, q.n, S->xs + X_DNORM, S->xs + X_FINAL);
     }
     S->greens(j->fd_d, j->x[0], j->x[1], j->x[2], j->x[3]);
     const size_t bytes = (size_t)S->B * sizeof(float);

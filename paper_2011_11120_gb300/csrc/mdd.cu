@@ -126,8 +126,8 @@ struct MddSolver {
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             copy_colsum<<<(Cu + 255) / 256, 256, 0, s>>>(p->nt, Cu, d, U, csU);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csU, Cu, part, nullptr);
-            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, resid, act + 1);
+            const SumSource q = colsum_source(csU, Cu, part, nullptr, s);
+            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, resid, act + 1);
         }
         // alpha_1 v_1 = G+^H u_1.  Each product's input is the unscaled spectrum the inverse
         // transform before it leaves (of v-hat, of u-hat); 1 / alpha and 1 / beta, which normalise
@@ -137,8 +137,8 @@ struct MddSolver {
         irfft(V, p->ns, C1(1.f), C1(0.f), csV, act + 1);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csV, Cv, part, act + 1);
-            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, act + 1);
+            const SumSource q = colsum_source(csV, Cv, part, act + 1, s);
+            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, act + 1);
             lsqr_xw_one_init<<<eg, 256, 0, s>>>(Bv, x, W, V, sc);
         }
         for (int it = 1; it <= niter; ++it) {
@@ -148,15 +148,15 @@ struct MddSolver {
             irfft(U, p->nr, CD(1.f, sc + S_INV_ALPHA), CD(1.f, sc + S_U_PREV), csU, a);
             {
                 LaunchScope ls(p, s, MDC_KC_SOLVER);
-                colsum_partials<<<PART_CTAS, 256, 0, s>>>(csU, Cu, part, a);
-                lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, a);
+                const SumSource q = colsum_source(csU, Cu, part, a, s);
+                lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a);
             }
             // v-hat <- G+^H u - beta v
             product(true, a);
             irfft(V, p->ns, CD(1.f, sc + S_INV_BETA), CD(1.f, sc + S_V_PREV), csV, a);
             LaunchScope ls(p, s, MDC_KC_SOLVER);
-            colsum_partials<<<PART_CTAS, 256, 0, s>>>(csV, Cv, part, a);
-            lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, part, PART_CTAS, a, act + it + 1, resid, iters, it, niter,
+            const SumSource q = colsum_source(csV, Cv, part, a, s);
+            lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a, act + it + 1, resid, iters, it, niter,
                                                         tol);
             lsqr_xw_one<<<eg, 256, 0, s>>>(Bv, x, W, V, sc, a);
         }
