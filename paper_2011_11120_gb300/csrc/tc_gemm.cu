@@ -14,7 +14,8 @@
 //            Re X'[s][n] = D[2s][2n] + D[2s+1][2n+1], Im X'[s][n] = D[2s][2n+1] - D[2s+1][2n].
 //            A = the SAME G buffer read MN-major (transposed operand); no second copy.
 //
-// One CTA computes a 128 x BN tile of D for one frequency: warp 0 streams A and B
+// 16-bit products of more than 64 columns run on SM pairs (tc_pair_kernel below).  Otherwise one CTA
+// computes a 128 x BN tile of D for one frequency: warp 0 streams A and B
 // tiles with TMA into a ring of 128-byte-swizzled shared-memory stages, warp 1 (one
 // thread) issues tcgen05.mma (M=128, N=BN, K=16, FP32 accumulation in TMEM), warps
 // 2-9 read the accumulator back with tcgen05.ld and write complex64 results.  B is
@@ -120,6 +121,66 @@ __device__ __forceinline__ bool epilogue_all(bool ok) {
         : "r"((uint32_t)ok)
         : "memory");
     return r != 0;
+}
+
+// Store 16 accumulator columns c0.. (8 complex output columns) of this warp's 32 rows of the tile (m0,
+// n0) of frequency k: scaled values go through a per-warp staging tile (rows padded to 20 floats, so both
+// the row-wise writes and the column-wise reads are conflict-free), then each store instruction writes 8
+// output rows x 64 contiguous bytes.  q: the warp's lane quarter; gs: its row's kernel scale (forward);
+// sgs: the tile's reciprocal column scales.
+template <bool ADJ>
+__device__ __forceinline__ void tc_emit16(const TcArgs& a, int k, int m0, int n0, int c0, int q, float gs,
+                                          const float* sgs, float* stg, const float* v) {
+    const int lane = threadIdx.x & 31;
+    const int nb = (n0 + c0) >> 1;
+    float w[16];
+    if (!ADJ) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float f = gs * sgs[(c0 >> 1) + j];
+            w[2 * j] = v[2 * j] * f;
+            w[2 * j + 1] = v[2 * j + 1] * f;
+        }
+    } else {
+        // rows 2s and 2s + 1 of the real product hold the two halves of output row s
+        float pv[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pv[j] = __shfl_xor_sync(0xffffffffu, v[j], 1);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float f = sgs[(c0 >> 1) + j];
+            w[2 * j] = (v[2 * j] + pv[2 * j + 1]) * f;
+            w[2 * j + 1] = (v[2 * j + 1] - pv[2 * j]) * f;
+        }
+    }
+    constexpr int NROWS = ADJ ? 16 : 32;
+    const int orow0 = ADJ ? (m0 + 32 * q) >> 1 : m0 + 32 * q;
+    if (!ADJ || (lane & 1) == 0) {
+        float* rowp = stg + (ADJ ? lane >> 1 : lane) * 20;
+#pragma unroll
+        for (int i4 = 0; i4 < 4; ++i4)
+            *reinterpret_cast<float4*>(rowp + 4 * i4) =
+                make_float4(w[4 * i4], w[4 * i4 + 1], w[4 * i4 + 2], w[4 * i4 + 3]);
+    }
+    __syncwarp();
+    const int cc = lane >> 3, n = nb + 2 * cc;
+#pragma unroll
+    for (int it = 0; it < NROWS / 8; ++it) {
+        const int rr = (lane & 7) + 8 * it, orow = orow0 + rr;
+        const float4 val = *reinterpret_cast<const float4*>(stg + rr * 20 + 4 * cc);
+        if (orow < a.nout && n < a.ncol &&
+            MDC_INB(((size_t)k * a.nout + orow) * a.ldo + a.voff_o + n, n + 1 < a.ncol ? 2 : 1,
+                    (long long)a.nf * a.nout * a.ldo, a.err, 130)) {
+            float2* dst = a.out + ((size_t)k * a.nout + orow) * a.ldo + a.voff_o + n;
+            if (n + 1 < a.ncol && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+                *reinterpret_cast<float4*>(dst) = val;
+            } else {
+                dst[0] = make_float2(val.x, val.y);
+                if (n + 1 < a.ncol) dst[1] = make_float2(val.z, val.w);
+            }
+        }
+    }
+    __syncwarp();
 }
 
 // Persistent CTA (one per SM): tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... with the
@@ -478,62 +539,8 @@ __global__ void __launch_bounds__(CVT ? TC_THREADS + TC_CVT_THREADS + 32 : TC_TH
             const int r = m0 + row;
             const float gs = (!ADJ && r < a.nout && MDC_INB((size_t)k * a.nr + r, 1, (long long)a.nf * a.nr, a.err, 132))
                                  ? a.gscale[(size_t)k * a.nr + r] : 1.f;
-            // Store 16 accumulator columns c0.. (8 complex output columns) of this warp's 32 rows:
-            // scaled values go through a per-warp staging tile (rows padded to 20 floats, so both
-            // the row-wise writes and the column-wise reads are conflict-free), then each store
-            // instruction writes 8 output rows x 64 contiguous bytes.
             float* stg = sig_s + 256 + (warp - 2) * (32 * 20);
-            auto emit = [&](int c0, const float* v) {
-                const int nb = (n0 + c0) >> 1;
-                float w[16];
-                if (!ADJ) {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float f = gs * sgs[(c0 >> 1) + j];
-                        w[2 * j] = v[2 * j] * f;
-                        w[2 * j + 1] = v[2 * j + 1] * f;
-                    }
-                } else {
-                    // rows 2s and 2s + 1 of the real product hold the two halves of output row s
-                    float pv[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) pv[j] = __shfl_xor_sync(0xffffffffu, v[j], 1);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float f = sgs[(c0 >> 1) + j];
-                        w[2 * j] = (v[2 * j] + pv[2 * j + 1]) * f;
-                        w[2 * j + 1] = (v[2 * j + 1] - pv[2 * j]) * f;
-                    }
-                }
-                constexpr int NROWS = ADJ ? 16 : 32;
-                const int orow0 = ADJ ? (m0 + 32 * q) >> 1 : m0 + 32 * q;
-                if (!ADJ || (lane & 1) == 0) {
-                    float* rowp = stg + (ADJ ? lane >> 1 : lane) * 20;
-#pragma unroll
-                    for (int i4 = 0; i4 < 4; ++i4)
-                        *reinterpret_cast<float4*>(rowp + 4 * i4) =
-                            make_float4(w[4 * i4], w[4 * i4 + 1], w[4 * i4 + 2], w[4 * i4 + 3]);
-                }
-                __syncwarp();
-                const int cc = lane >> 3, n = nb + 2 * cc;
-#pragma unroll
-                for (int it = 0; it < NROWS / 8; ++it) {
-                    const int rr = (lane & 7) + 8 * it, orow = orow0 + rr;
-                    const float4 val = *reinterpret_cast<const float4*>(stg + rr * 20 + 4 * cc);
-                    if (orow < a.nout && n < a.ncol &&
-                        MDC_INB(((size_t)k * a.nout + orow) * a.ldo + a.voff_o + n, n + 1 < a.ncol ? 2 : 1,
-                                (long long)a.nf * a.nout * a.ldo, a.err, 130)) {
-                        float2* dst = a.out + ((size_t)k * a.nout + orow) * a.ldo + a.voff_o + n;
-                        if (n + 1 < a.ncol && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-                            *reinterpret_cast<float4*>(dst) = val;
-                        } else {
-                            dst[0] = make_float2(val.x, val.y);
-                            if (n + 1 < a.ncol) dst[1] = make_float2(val.z, val.w);
-                        }
-                    }
-                }
-                __syncwarp();
-            };
+            auto emit = [&](int c0, const float* v) { tc_emit16<ADJ>(a, k, m0, n0, c0, q, gs, sgs, stg, v); };
             bool ok = true;
             if constexpr (SPLIT) {
                 // sum the chunks' partial accumulators in float32 registers, then store
@@ -591,6 +598,241 @@ __global__ void __launch_bounds__(CVT ? TC_THREADS + TC_CVT_THREADS + 32 : TC_TH
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, SC::TCOLS);
+    }
+}
+
+// ------------------------------------------------------------------ 16-bit products by SM pairs
+// With 256-column tiles the kernel above is bound by the delivery of its operands: 48 KB per 64 reduction
+// elements into each SM (18 TB/s from L2 over 152 SMs) and twice that through shared memory.  Here the
+// two CTAs of a cluster compute one 256 x 256 tile with cta_group::2 MMAs: each loads 128 rows of A and
+// half of B (plain TMA loads into its own shared memory, no multicast), 32 KB, and keeps the accumulator
+// of its 128 rows in its own TMEM.  Forward / adjoint, single CTAs and pairs: 128 columns on 8281^2 x 40
+// 2.21 / 2.11 and 1.83 / 1.78 ms; 512 columns on 1681^2 x 150 1.21 / 1.49 and 1.13 / 1.15 ms (1.54
+// PFLOP/s, 0.88 of the measured sustained bfloat16 rate; what bounds it now is power).  Narrower tiles
+// stay on single CTAs: they are bound by the kernel's bytes from HBM.
+//
+// The leader (rank 0) owns the full barriers (both CTAs' loads report there) and issues the MMAs; their
+// commits release the stage and hand over the accumulator in both CTAs.  Both epilogues report the
+// accumulator empty to the leader.  Every wait is bounded as in tc_gemm_kernel; both CTAs always reach
+// the closing cluster barrier, before which the leader has seen all copies land and all MMAs complete.
+constexpr int PR_BN = 256;
+constexpr int PR_STAGES = 6;
+constexpr uint32_t PR_A_BYTES = TC_BM * 128, PR_B_BYTES = (PR_BN / 2) * 128, PR_STAGE = PR_A_BYTES + PR_B_BYTES;
+
+// Bound on the leader's wait for each of the last copies: they land in microseconds, but the barrier
+// also counts the other CTA's, which may have given up.
+constexpr unsigned long long PR_DRAIN_NS = 20000000ull;
+
+constexpr size_t pair_smem_bytes() {
+    // + alignment, barriers, two 128-float column-scale buffers, eight staging tiles
+    return (size_t)PR_STAGES * PR_STAGE + 1024 + 256 + 1024 + 8 * 32 * 20 * 4;
+}
+
+__device__ __forceinline__ uint32_t cta_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t leader_addr(uint32_t addr) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A load into this CTA's shared memory that reports to a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
+                                                 int c2) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+        "l"((unsigned long long)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+__device__ __forceinline__ void umma_f16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+// Completion of this thread's MMAs arrives on the barrier at this offset in both CTAs of the pair.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+    const uint16_t both = 3;
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        "h"(both)
+        : "memory");
+}
+
+template <bool ADJ>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
+    tc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a,
+                   uint32_t idesc, const int* active, int n_tiles_n, int n_tiles_m, int n_tiles) {
+    if (active && *active == 0) return;              // the same answer in both CTAs
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t raw = su32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    unsigned char* gbase = smem_raw + (base - raw);
+    // full[S], empty[S], acc_full[2], acc_empty[2], drain, tmem slot; column scales 256 bytes on
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + PR_STAGES * PR_STAGE);
+    const uint32_t full0 = su32(bars), empty0 = full0 + 8 * PR_STAGES;
+    const uint32_t accf0 = empty0 + 8 * PR_STAGES, acce0 = accf0 + 16, drain0 = acce0 + 16;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * PR_STAGES + 5);
+    static_assert(2 * PR_STAGES + 6 <= 32, "barrier space");
+    float* sig_s = reinterpret_cast<float*>(bars + 32);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cta_rank();
+    const int t_first = (int)(blockIdx.x >> 1), t_stride = (int)(gridDim.x >> 1);
+    const unsigned long long wl = a.wait_ns;
+
+    if (threadIdx.x == 32) {
+        for (int i = 0; i < PR_STAGES; ++i) {
+            mbar_init(full0 + 8 * i, 1);
+            mbar_init(empty0 + 8 * i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(accf0 + 8 * i, 1);
+            mbar_init(acce0 + 8 * i, 16);            // eight epilogue warps of each CTA
+        }
+        mbar_init(drain0, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
+                     "r"(2 * PR_BN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                              // both CTAs' barriers exist
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const int per_freq = n_tiles_n * n_tiles_m;
+    // tile t -> frequency k, this CTA's first row m0, first column n0
+    auto coords = [&](int t, int& k, int& m0, int& n0) {
+        k = t / per_freq;
+        const int rem = t - k * per_freq;
+        const int mt = rem / n_tiles_n;
+        m0 = mt * 2 * TC_BM + (int)rank * TC_BM;
+        n0 = (rem - mt * n_tiles_n) * PR_BN;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            long g = 0;
+            bool ok = true;
+            for (int tile = t_first; tile < n_tiles && ok; tile += t_stride) {
+                int k, m0, n0;
+                coords(tile, k, m0, n0);
+                for (int kb = 0; kb < a.kstages; ++kb, ++g) {
+                    const int s = (int)(g % PR_STAGES);
+                    if (g >= PR_STAGES &&
+                        !mbar_wait(empty0 + 8 * s, (uint32_t)(g / PR_STAGES - 1) & 1, a.err, 41, wl)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t sa = base + s * PR_STAGE, sb = sa + PR_A_BYTES;
+                    const uint32_t bar = leader_addr(full0 + 8 * s);
+                    if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * PR_STAGE);      // both CTAs' bytes
+                    if (!ADJ) {
+                        tma_load_3d_pair(sa, &tmA, bar, kb * TC_BK, m0, k);
+                    } else {
+                        tma_load_3d_pair(sa, &tmA, bar, m0, kb * TC_BK, k);
+                        tma_load_3d_pair(sa + PR_A_BYTES / 2, &tmA, bar, m0 + 64, kb * TC_BK, k);
+                    }
+                    tma_load_3d_pair(sb, &tmB, bar, kb * TC_BK, n0 + (int)rank * (PR_BN / 2), k);
+                }
+            }
+            // both CTAs' copies have landed (they all report here) before either CTA can exit
+            if (rank == 0)
+                for (long q = g > PR_STAGES ? g - PR_STAGES : 0; q < g; ++q)
+                    mbar_wait(full0 + 8 * (int)(q % PR_STAGES), (uint32_t)(q / PR_STAGES) & 1, a.err, 42, PR_DRAIN_NS);
+        }
+    } else if (warp == 1) {
+        if (rank == 0 && lane == 0) {
+            long g = 0, i = 0;
+            bool ok = true;
+            for (int tile = t_first; tile < n_tiles && ok; tile += t_stride, ++i) {
+                const int buf = (int)(i & 1);
+                if (i >= 2 && !mbar_wait(acce0 + 8 * buf, (uint32_t)((i >> 1) - 1) & 1, a.err, 43, wl)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(buf * PR_BN);
+                for (int kb = 0; kb < a.kstages; ++kb, ++g) {
+                    const int s = (int)(g % PR_STAGES);
+                    if (!mbar_wait(full0 + 8 * s, (uint32_t)(g / PR_STAGES) & 1, a.err, 44, wl)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t sa = base + s * PR_STAGE, sb = sa + PR_A_BYTES;
+#pragma unroll
+                    for (int kk = 0; kk < TC_BK / 16; ++kk) {
+                        const uint64_t ad = sdesc(sa + (ADJ ? kk * 2048 : kk * 32), ADJ ? PR_A_BYTES / 2 : 16, 1024);
+                        umma_f16_pair(d, ad, sdesc(sb + kk * 32, 16, 1024), idesc, (kb | kk) != 0 ? 1u : 0u);
+                    }
+                    umma_commit_pair(empty0 + 8 * s);
+                }
+                umma_commit_pair(accf0 + 8 * buf);
+            }
+            // every MMA has completed before either CTA frees TMEM
+            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain0)
+                         : "memory");
+            mbar_wait(drain0, 0, a.err, 45, TC_DRAIN_NS);
+        }
+    } else {
+        const int q = warp & 3;                  // TMEM lane quarter of this warp
+        constexpr int BH = PR_BN / 2;
+        const int cbeg = ((warp - 2) >> 2) * BH;
+        float* stg = sig_s + 256 + (warp - 2) * (32 * 20);
+        long i = 0;
+        for (int tile = t_first; tile < n_tiles; tile += t_stride, ++i) {
+            int k, m0, n0;
+            coords(tile, k, m0, n0);
+            const int buf = (int)(i & 1);
+            float* sgs = sig_s + buf * 128;      // this tile's reciprocal column scales (alternating)
+            {
+                const int e = threadIdx.x - 64, n = (n0 >> 1) + e;
+                if (e < PR_BN / 2)
+                    sgs[e] = n < a.ncol && MDC_INB((size_t)k * a.ncol + n, 1, (long long)a.nf * a.ncol, a.err, 151)
+                                 ? a.inv_sigma[(size_t)k * a.ncol + n] : 0.f;
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+            }
+            const int r = m0 + q * 32 + lane;
+            const float gs = (!ADJ && r < a.nout && MDC_INB((size_t)k * a.nr + r, 1, (long long)a.nf * a.nr, a.err, 152))
+                                 ? a.gscale[(size_t)k * a.nr + r] : 1.f;
+            if (!epilogue_all(mbar_wait(accf0 + 8 * buf, (uint32_t)(i >> 1) & 1, a.err, 46, wl))) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * PR_BN);
+#pragma unroll 1
+            for (int c0 = cbeg; c0 < cbeg + BH; c0 += 16) {
+                uint32_t v[16];
+                tmem_ld16(taddr + c0, v);
+                float f[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+                tc_emit16<ADJ>(a, k, m0, n0, c0, q, gs, sgs, stg, f);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                                 leader_addr(acce0 + 8 * buf))
+                             : "memory");
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                          // no CTA leaves while the other may signal or use it
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * PR_BN) : "memory");
     }
 }
 
@@ -1173,6 +1415,42 @@ bool launch_tc(const CUtensorMap* maps, const TcArgs& a, uint32_t idesc, dim3 gr
     return true;
 }
 
+// The SM-pair kernel over (column tiles, row-pair tiles, frequencies); false if no cluster can run.
+template <bool ADJ>
+bool launch_pair(const CUtensorMap* maps, const TcArgs& a, uint32_t idesc, dim3 grid, cudaStream_t s,
+                 const int* active) {
+    static SmemLimit attr;
+    static std::atomic<int> clusters[64];            // co-resident pairs per device, + 1
+    constexpr size_t smem = pair_smem_bytes();
+    attr.ensure(tc_pair_kernel<ADJ>, (int)smem);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    int n = clusters[dev].load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2);
+        cfg.blockDim = dim3(TC_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 2;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<ADJ>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        clusters[dev].store(n + 1, std::memory_order_relaxed);
+    }
+    if (n < 1) return false;
+    const int n_tiles = (int)grid.x * (int)grid.y * (int)grid.z;
+    const int pairs = n_tiles < n ? n_tiles : n;
+    tc_pair_kernel<ADJ><<<2 * pairs, TC_THREADS, smem, s>>>(maps[0], maps[1], a, idesc, active, (int)grid.x,
+                                                            (int)grid.y, n_tiles);
+    return true;
+}
+
 // MDC_E4M3_SWAP=0 in the environment keeps narrow E4M3 forward products on the widening kernel
 // (for comparisons).
 bool f8_swap_allowed() {
@@ -1308,7 +1586,9 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
     const size_t blo = plane * 2;                                          // lo plane of B (bytes)
     // row tiles of the product (kernel rows forward; 2 * ldg interleaved reals adjoint)
     const int mrows = adjoint ? (int)(kp / TC_BM) : (p->nr + TC_BM - 1) / TC_BM;
-    const int bbox = bn;
+    // 256-column tiles of the 16-bit copies run on SM pairs, each CTA loading half of a tile's B rows
+    const bool pair = bn == PR_BN && !split && !e4m3;
+    const int bbox = pair ? bn / 2 : bn;
     bool ok = true;
     const uint64_t ab = e4m3 ? 1 : 2;         // bytes per real of the kernel copy
     // E4M3 byte tiles: forward 128 rows x 128 bytes for B tiles of <= 64 columns (two reduction
@@ -1351,6 +1631,11 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
                            ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
     dim3 grid((unsigned)(rows_pad / bn), (unsigned)mrows, (unsigned)p->nf);
     if (scoped) scope.emplace(p, s, adjoint ? MDC_KC_PRODUCT_ADJ : MDC_KC_PRODUCT_FWD);
+    if (pair) {
+        const uint32_t id2 = (idesc & ~(0x1fu << 24)) | ((uint32_t)(2 * TC_BM >> 4) << 24);      // M = 256
+        const dim3 g2(grid.x, (grid.y + 1) / 2, grid.z);
+        return adjoint ? launch_pair<true>(maps, a, id2, g2, s, active) : launch_pair<false>(maps, a, id2, g2, s, active);
+    }
 #define MDC_TC_LAUNCH(ADJV, BV, SPV)                                                             \
     if (e4m3)                                                                                    \
         launched = launch_tc<ADJV, BV, false, true>(maps, a, idesc, grid, s, active);               \
@@ -1359,9 +1644,8 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
 #define MDC_TC_CASE(BNV)                                                                   \
     case BNV:                                                                              \
         if (split) {                                                                       \
-            constexpr int BS = BNV > 128 ? 128 : BNV;                                      \
-            if (adjoint) { MDC_TC_LAUNCH(true, BS, true) }                                 \
-            else { MDC_TC_LAUNCH(false, BS, true) }                                        \
+            if (adjoint) { MDC_TC_LAUNCH(true, BNV, true) }                                \
+            else { MDC_TC_LAUNCH(false, BNV, true) }                                       \
         } else {                                                                           \
             if (adjoint) { MDC_TC_LAUNCH(true, BNV, false) }                               \
             else { MDC_TC_LAUNCH(false, BNV, false) }                                      \
@@ -1372,7 +1656,10 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
         MDC_TC_CASE(32)
         MDC_TC_CASE(64)
         MDC_TC_CASE(128)
-        MDC_TC_CASE(256)
+        case 256:                                    // E4M3 (the 16-bit copies run on pairs, split has no 256)
+            launched = adjoint ? launch_tc<true, 256, false, true>(maps, a, idesc, grid, s, active)
+                               : launch_tc<false, 256, false, true>(maps, a, idesc, grid, s, active);
+            break;
     }
 #undef MDC_TC_CASE
 #undef MDC_TC_LAUNCH
