@@ -164,7 +164,6 @@ template <int N1, int N2, bool WIN, bool X2, int PP>
 __global__ void __launch_bounds__(FFT_THREADS, 2) rfft4_kernel(RfftArgs a) {
     using F = FourStep<N1, N2, PP>;
     constexpr int NT = F::NT, CT = F::CT;
-    if (a.active && *a.active == 0) return;
     extern __shared__ __align__(16) float2 sm2[];
     float2* tw = sm2;                  // W_NT^m for the whole period m < NT
     float2* z = sm2 + NT;
@@ -174,6 +173,8 @@ __global__ void __launch_bounds__(FFT_THREADS, 2) rfft4_kernel(RfftArgs a) {
         tw[i] = w;
         tw[i + NT / 2] = make_float2(-w.x, -w.y);
     }
+    pdl_wait();                                           // the input; the twiddles above are constants
+    if (a.active && *a.active == 0) return;
     // First pass straight from global memory: task (j, n2) loads the column pair (c0 + 2j, c0 + 2j + 1)
     // at rows n1 * N2 + n2 (a warp reads whole 64- or 128-byte row segments), applies the window,
     // transforms over n1 in registers, twiddles, and writes the tile; only the second pass goes through
@@ -706,7 +707,7 @@ void rfft4_go(mdc_plan* p, const RfftArgs& a, cudaStream_t s) {
     static SmemLimit attr;
     attr.ensure(rfft4_kernel<N1, N2, WIN, X2, PP>, (int)F::smem_full);
     LaunchScope ls(p, s, MDC_KC_RFFT);
-    rfft4_kernel<N1, N2, WIN, X2, PP><<<(a.C + F::CT - 1) / F::CT, FFT_THREADS, F::smem_full, s>>>(a);
+    launch_pdl(rfft4_kernel<N1, N2, WIN, X2, PP>, dim3((a.C + F::CT - 1) / F::CT), FFT_THREADS, F::smem_full, s, a);
 }
 
 template <int N1, int N2>

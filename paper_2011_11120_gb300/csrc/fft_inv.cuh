@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(FFT_THREADS, MODE == 1 ? 3 : 2) irfft4_kernel(
     static_assert(!(FUSE && PLAIN), "the fused forward transform follows the general epilogue");
     using F = FourStep<N1, N2, PP>;
     constexpr int NT = F::NT, CT = F::CT, P = F::P;
-    if (a.active && *a.active == 0) return;
     extern __shared__ __align__(16) float2 sm2[];
     float2* tw = sm2;                  // exp(+2 pi i m / NT) for the whole period
     float2* z = sm2 + NT;
@@ -44,6 +43,8 @@ __global__ void __launch_bounds__(FFT_THREADS, MODE == 1 ? 3 : 2) irfft4_kernel(
         tw[i] = make_float2(w.x, -w.y);
         tw[i + NT / 2] = make_float2(-w.x, w.y);
     }
+    pdl_wait();                                          // the spectrum; the twiddles above are constants
+    if (a.active && *a.active == 0) return;
     // every thread keeps one column pair (FFT_THREADS is a multiple of P)
     const int j = threadIdx.x % P, c = c0 + 2 * j;
     const bool has0 = c < a.C, has1 = c + 1 < a.C;
@@ -104,9 +105,11 @@ __global__ void __launch_bounds__(FFT_THREADS, MODE == 1 ? 3 : 2) irfft4_kernel(
                 const float s = mir ? -sg : sg;          // sign of the imaginary parts
 #pragma unroll
                 for (int u = 0; u < BA; ++u) {
-                    float ay = s * q[u].y, by = s * q[u].w;
+                    // each value scaled, then joined (a solve's Green's functions show every rounding)
+                    const float si = s * isc;
+                    float ay = si * q[u].y, by = si * q[u].w;
                     if ((b + u == 0 || b + u == N1 / 2) && n2 == 0) ay = by = 0.f;     // DC, Nyquist
-                    r[b + u] = make_float2(isc * (q[u].x - by), isc * (ay + q[u].z));
+                    r[b + u] = make_float2(__fsub_rn(isc * q[u].x, by), __fadd_rn(ay, isc * q[u].z));
                 }
             }
             reg_fft<N1, true>(r);
@@ -268,7 +271,7 @@ void irfft4_go(mdc_plan* p, const IrfftArgs& a, cudaStream_t s) {
     static SmemLimit attr;
     attr.ensure(irfft4_kernel<N1, N2, MODE, PP, FUSE, V2>, (int)smem);
     LaunchScope ls(p, s, MDC_KC_IRFFT);
-    irfft4_kernel<N1, N2, MODE, PP, FUSE, V2><<<(a.C + F::CT - 1) / F::CT, FFT_THREADS, smem, s>>>(a);
+    launch_pdl(irfft4_kernel<N1, N2, MODE, PP, FUSE, V2>, dim3((a.C + F::CT - 1) / F::CT), FFT_THREADS, smem, s, a);
 }
 
 template <int N1, int N2, int PP, bool V2>

@@ -144,7 +144,7 @@ struct Solver {
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             const SumSource q = colsum_source(csU, 2 * C, part, nullptr, s);
-            norm_store<<<1, RED_THREADS, 0, s>>>(q.v, q.n, xs + X_DNORM);
+            launch_pdl(norm_store, 1, RED_THREADS, 0, s, q.v, q.n, xs + X_DNORM);
         }
         if (D1()) {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
@@ -187,13 +187,13 @@ struct Solver {
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             const SumSource q = colsum_source(csU, 2 * C, part, nullptr, s);
-            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, resid0, act0 + 1);
+            launch_pdl(lsqr_init_beta, 1, RED_THREADS, 0, s, sc, q.v, q.n, resid0, act0 + 1);
         }
         apply_MH(act0 + 1, zero);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             const SumSource q = colsum_source(csV, 2 * C, part, act0 + 1, s);
-            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, act0 + 1);
+            launch_pdl(lsqr_init_alpha, 1, RED_THREADS, 0, s, sc, q.v, q.n, act0 + 1);
         }
         LaunchScope ls(p, s, MDC_KC_SOLVER);
         if (zero_x) lsqr_xw_init<<<eg, 256, 0, s>>>(B, x1, x2, W1(), W2(), V1(), V2(), sc);
@@ -219,7 +219,7 @@ struct Solver {
               nullptr, nullptr, nv, cut, 1);
         LaunchScope ls(p, s, MDC_KC_SOLVER);
         const SumSource q = colsum_source(csU, 2 * C, part, a, s);
-        lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a);
+        launch_pdl(lsqr_beta, 1, RED_THREADS, 0, s, sc, q.v, q.n, a);
     }
     //   v-hat <- M^H u - beta v
     void iter_adj_pre(const int*) {}
@@ -235,7 +235,7 @@ struct Solver {
               a, x2, W2(), fuse_v ? 0 : -1, nullptr, 0);
         LaunchScope ls(p, s, MDC_KC_SOLVER);
         const SumSource q = colsum_source(csV, 2 * C, part, a, s);
-        lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a, act0 + it + 1, resid0, itp, it,
+        launch_pdl(lsqr_alpha_rotate, 1, RED_THREADS, 0, s, sc, q.v, q.n, a, act0 + it + 1, resid0, itp, it,
                                                     niter, tol);
     }
     // The last rotation's pending x step (once per solve, after its last iteration).
@@ -340,7 +340,7 @@ void solve_body(Solver& S, const float* fd, int niter, int nref, int niter_ref, 
         S.residual_pass(fm, fmp);
         LaunchScope ls(S.p, S.s, MDC_KC_SOLVER);
         const SumSource q = colsum_source(S.csU, 2 * S.C, S.part, nullptr, S.s);
-        norm_ratio<<<1, RED_THREADS, 0, S.s>>>(q.v, q.n, S.xs + X_DNORM, S.xs + X_FINAL);
+        launch_pdl(norm_ratio, 1, RED_THREADS, 0, S.s, q.v, q.n, S.xs + X_DNORM, S.xs + X_FINAL);
     }
     if (gm || gp) S.greens(fd, fm, fmp, gm, gp);
 }
@@ -789,7 +789,7 @@ void finish_job(mdc_server* v, ServeJob* j) {
     {
         LaunchScope ls(v->p, v->s, MDC_KC_SOLVER);
         const SumSource q = colsum_source(S->csU, 2 * S->C, S->part, nullptr, v->s);
-        norm_ratio<<<1, RED_THREADS, 0, v->s>>>(q.v, q.n, S->xs + X_DNORM, S->xs + X_FINAL);
+        launch_pdl(norm_ratio, 1, RED_THREADS, 0, v->s, q.v, q.n, S->xs + X_DNORM, S->xs + X_FINAL);
     }
     S->greens(j->fd_d, j->x[0], j->x[1], j->x[2], j->x[3]);
     const size_t bytes = (size_t)S->B * sizeof(float);

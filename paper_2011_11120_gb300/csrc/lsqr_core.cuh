@@ -53,6 +53,7 @@ __device__ double block_sum(const double* v, int n) {
 constexpr int PART_CTAS = 304;
 __global__ void __launch_bounds__(256) colsum_partials(const double* __restrict__ cs, int n,
                                                        double* __restrict__ part, const int* act) {
+    pdl_wait();
     if (act && *act == 0) return;
     __shared__ double red[256];
     const int chunk = (n + PART_CTAS - 1) / PART_CTAS;
@@ -83,13 +84,14 @@ struct SumSource {
 };
 inline SumSource colsum_source(const double* cs, int n, double* part, const int* act, cudaStream_t s) {
     if (n <= DIRECT_SUM) return {cs, n};
-    colsum_partials<<<PART_CTAS, 256, 0, s>>>(cs, n, part, act);
+    launch_pdl(colsum_partials, PART_CTAS, 256, 0, s, cs, n, part, act);
     return {part, PART_CTAS};
 }
 
 // beta_1 = ||d||, u_1 = d / beta_1 (Paige-Saunders initialisation).
 __global__ void __launch_bounds__(RED_THREADS) lsqr_init_beta(double* sc, const double* cs, int n,
                                                               double* resid, int* act1) {
+    pdl_wait();
     const double b = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) {
         sc[S_BETA] = b;
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(RED_THREADS) lsqr_init_beta(double* sc, const 
 // alpha_1 v_1 = M^H u_1, w_1 = v_1, rhobar_1 = alpha_1.
 __global__ void __launch_bounds__(RED_THREADS) lsqr_init_alpha(double* sc, const double* cs, int n,
                                                                int* act1) {
+    pdl_wait();
     if (*act1 == 0) return;
     const double a = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) {
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(RED_THREADS) lsqr_init_alpha(double* sc, const
 // After u-hat = M v - alpha u: beta = ||u-hat||, coefficients for the M^H step.
 __global__ void __launch_bounds__(RED_THREADS) lsqr_beta(double* sc, const double* cs, int n,
                                                          const int* act) {
+    pdl_wait();
     if (*act == 0) return;
     const double b = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) {
@@ -136,6 +140,7 @@ __global__ void __launch_bounds__(RED_THREADS) lsqr_alpha_rotate(double* sc, con
                                                                  const int* act, int* act_next,
                                                                  double* resid, int* iters, int it,
                                                                  int niter, double tol) {
+    pdl_wait();
     if (*act == 0) return;
     double a = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) {
@@ -216,10 +221,12 @@ int elementwise_grid(int64_t n) {
 
 // sqrt(sum of column sums) / reference norm, written to out (the FP64 residual check).
 __global__ void __launch_bounds__(RED_THREADS) norm_ratio(const double* cs, int n, const double* ref, double* out) {
+    pdl_wait();
     const double v = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) *out = (*ref > 0.0) ? v / *ref : v;
 }
 __global__ void __launch_bounds__(RED_THREADS) norm_store(const double* cs, int n, double* out) {
+    pdl_wait();
     const double v = sqrt(block_sum(cs, n));
     if (threadIdx.x == 0) *out = v;
 }

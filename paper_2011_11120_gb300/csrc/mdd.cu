@@ -127,7 +127,7 @@ struct MddSolver {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             copy_colsum<<<(Cu + 255) / 256, 256, 0, s>>>(p->nt, Cu, d, U, csU);
             const SumSource q = colsum_source(csU, Cu, part, nullptr, s);
-            lsqr_init_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, resid, act + 1);
+            launch_pdl(lsqr_init_beta, 1, RED_THREADS, 0, s, sc, q.v, q.n, resid, act + 1);
         }
         // alpha_1 v_1 = G+^H u_1.  Each product's input is the unscaled spectrum the inverse
         // transform before it leaves (of v-hat, of u-hat); 1 / alpha and 1 / beta, which normalise
@@ -138,7 +138,7 @@ struct MddSolver {
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             const SumSource q = colsum_source(csV, Cv, part, act + 1, s);
-            lsqr_init_alpha<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, act + 1);
+            launch_pdl(lsqr_init_alpha, 1, RED_THREADS, 0, s, sc, q.v, q.n, act + 1);
             lsqr_xw_one_init<<<eg, 256, 0, s>>>(Bv, x, W, V, sc);
         }
         for (int it = 1; it <= niter; ++it) {
@@ -149,14 +149,14 @@ struct MddSolver {
             {
                 LaunchScope ls(p, s, MDC_KC_SOLVER);
                 const SumSource q = colsum_source(csU, Cu, part, a, s);
-                lsqr_beta<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a);
+                launch_pdl(lsqr_beta, 1, RED_THREADS, 0, s, sc, q.v, q.n, a);
             }
             // v-hat <- G+^H u - beta v
             product(true, a);
             irfft(V, p->ns, CD(1.f, sc + S_INV_BETA), CD(1.f, sc + S_V_PREV), csV, a);
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             const SumSource q = colsum_source(csV, Cv, part, a, s);
-            lsqr_alpha_rotate<<<1, RED_THREADS, 0, s>>>(sc, q.v, q.n, a, act + it + 1, resid, iters, it, niter,
+            launch_pdl(lsqr_alpha_rotate, 1, RED_THREADS, 0, s, sc, q.v, q.n, a, act + it + 1, resid, iters, it, niter,
                                                         tol);
             lsqr_xw_one<<<eg, 256, 0, s>>>(Bv, x, W, V, sc, a);
         }

@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_adj_c64(
     const float4* __restrict__ G, int ldg, int nr, int ns,
     const float2* __restrict__ Yin, int ldi, int voff_i,
     float2* __restrict__ Xout, int ldo, int voff_o, const int* active, int* err) {
+    pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 ys[];   // [nr][NVC], then reduction space
     const int k = blockIdx.y;
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd(
     float2* __restrict__ Y, int ldo, int voff_o, const int* active, int64_t lo, int* err) {
     using FR = FwdRows<FMT, NVC, SHAPE>;
     constexpr int CPV = Fmt<FMT>::CPV, RB = FR::RB, W = GEMV_THREADS / 32;
+    pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 xs[];   // [NVC][CPV][nvec]
     const int k = blockIdx.y;
@@ -314,6 +316,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_adj(
     constexpr int CPV = Fmt<FMT>::CPV;
     constexpr int TILE = 32 * CPV;
     constexpr int W = GEMV_THREADS / 32;
+    pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 ys[];   // [nr][NVC], then reduction space
     const int k = blockIdx.y;
@@ -423,6 +426,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_chunked(
     constexpr int CHV = FwdChunk<FMT, NVC>::CHV;
     constexpr int W = GEMV_THREADS / 32;
     constexpr int NB = FWD_CHUNK_ROWS / (W * RB);      // batches of RB rows per warp
+    pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 xs[];   // [NVC][CPV][CHV]
     const int k = blockIdx.y;
@@ -475,6 +479,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_adj_chunked(
     constexpr int TILE = 32 * CPV;
     constexpr int W = GEMV_THREADS / 32;
     constexpr int CHR = AdjChunk<NVC>::CHR;
+    pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 ys[];   // [CHR][NVC], then reduction space
     const int k = blockIdx.y;
@@ -726,16 +731,16 @@ void gemv_fwd_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
     if (smem > (size_t)GEMV_STAGE_MAX && gemv_chunk_allowed()) {
         constexpr size_t csmem = (size_t)Fmt<FMT>::CPV * FwdChunk<FMT, NVC>::CHV * NVC * sizeof(float2);
         dim3 grid((p->nr + FWD_CHUNK_ROWS - 1) / FWD_CHUNK_ROWS, p->nf);
-        gemv_fwd_chunked<FMT, NVC><<<grid, GEMV_THREADS, csmem, s>>>(
-            reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out,
-            ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+        launch_pdl(gemv_fwd_chunked<FMT, NVC>, grid, GEMV_THREADS, csmem, s, reinterpret_cast<const uint4*>(p->G),
+                   (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
+                   p->err_flag);
         return;
     }
     dim3 grid((p->nr + FWD_ROWS_PER_CTA - 1) / FWD_ROWS_PER_CTA, p->nf);
     auto go = [&](auto kern, SmemLimit& attr) {
         attr.ensure(kern, 220 * 1024);
-        kern<<<grid, GEMV_THREADS, smem, s>>>(reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale,
-                                              in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+        launch_pdl(kern, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr,
+                   p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
     };
     if constexpr ((FMT == MDC_C64 || FMT == MDC_C32S) && NVC == 1) {
         if (p->ldg > LONG_ROW) {
@@ -760,9 +765,9 @@ void gemv_adj_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
         static SmemLimit cattr;
         cattr.ensure(gemv_adj_chunked<FMT, NVC>, 220 * 1024);
         dim3 grid((unsigned)((p->ldg + TILE - 1) / TILE), p->nf);
-        gemv_adj_chunked<FMT, NVC><<<grid, GEMV_THREADS, csmem, s>>>(
-            reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out,
-            ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+        launch_pdl(gemv_adj_chunked<FMT, NVC>, grid, GEMV_THREADS, csmem, s, reinterpret_cast<const uint4*>(p->G),
+                   (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
+                   p->err_flag);
         return;
     }
     if (smem < red) smem = red;
@@ -772,14 +777,13 @@ void gemv_adj_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
     if constexpr (FMT == MDC_C64) {
         static SmemLimit attr64;
         attr64.ensure(gemv_adj_c64<NVC>, 220 * 1024);
-        gemv_adj_c64<NVC><<<grid, GEMV_THREADS, smem, s>>>(
-            reinterpret_cast<const float4*>(p->G), (int)p->ldg, p->nr, p->ns, in, ldi, voff_i, out, ldo,
-            voff_o, active, p->err_flag);
+        launch_pdl(gemv_adj_c64<NVC>, grid, GEMV_THREADS, smem, s, reinterpret_cast<const float4*>(p->G),
+                   (int)p->ldg, p->nr, p->ns, in, ldi, voff_i, out, ldo, voff_o, active, p->err_flag);
         return;
     }
-    gemv_adj<FMT, NVC><<<grid, GEMV_THREADS, smem, s>>>(
-        reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out,
-        ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+    launch_pdl(gemv_adj<FMT, NVC>, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G),
+                   (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
+                   p->err_flag);
 }
 
 bool gemv_fits(const mdc_plan* p, bool adjoint, int ncol, int cpv) {
