@@ -111,6 +111,8 @@ def _check(status: int, where: str) -> None:
 
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
+        if torch.cuda.is_initialized():              # the raw handle, without a Stream object per call
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
