@@ -316,7 +316,7 @@ def run_redatum(args, dev):
     t_plain, err, plain = None, None, {"iters": None}
     if not args.redatum_skip_fp32:
         t0 = time.perf_counter()
-        plain = plain_op.marchenko(cut, fd, niter)     # complex64 SIMT operator, one job, no refinement
+        plain = plain_op.marchenko(cut, fd, niter)     # complex64 operator, one job, no refinement
         t_plain = time.perf_counter() - t0
         fm = out["f_minus"].double()
         err = float((fm - plain["f_minus"].double()).norm() / plain["f_minus"].double().norm())
@@ -357,7 +357,7 @@ def run_redatum(args, dev):
 def run_mdd(args, dev):
     """Multi-dimensional deconvolution (Eq. 8): a stand-in down-going Green's function G+ between
     the 61 x 61 surface grid and a 29 x 29 lattice of focusing points (nt=1024, nfmax=200), one
-    batch of 20 virtual sources per LSQR solve, with complex64 (FP32 SIMT products), split FP16
+    batch of 20 virtual sources per LSQR solve, with complex64 (float32-accurate products), split FP16
     (float32-accurate tensor-core products) and FP16 (tensor cores) kernel copies; the tensor-core
     results are compared with the complex64 one."""
     import torch
@@ -470,9 +470,6 @@ def run_precision(args, dev):
     return out
 
 
-FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz max SM clock
-
-
 def run_small(args, dev):
     """The small workload (441 x 441, nt=256, nfmax=64, nv=1; complex64 kernel 99.6 MB, smaller than
     L2): forward+adjoint pairs timed one by one (CUDA events around each pair, median of
@@ -541,7 +538,7 @@ def run_small(args, dev):
 def run_batched64(args, dev):
     """The paper-scale kernel (3721 x 3721, nt=1024, nfmax=200) with nv = 64 random focusing points:
     every product is a dense GEMM per frequency (1.42 TFLOP).  Split FP16 storage (three FP16
-    tensor-core products per GEMM, float32-level accuracy) against complex64 on the FP32 SIMT GEMM;
+    tensor-core products per GEMM) against complex64 (six bfloat16 ones, float32 accuracy);
     sampled rows/columns against the FP64 oracle."""
     import torch
     import paper_2011_11120_gb300 as mdc
@@ -597,10 +594,11 @@ def run_batched64(args, dev):
                                "achieved": issued, "peak": pk, "unit": "TFLOP/s", "frac": issued / pk,
                                "peak_kind": kind, "note": "achieved counts the three tensor-core products issued"}
         else:
-            res["roofline"] = {"bound": "alu", "kernel": "cgemm_simt (FP32 FMA)", "achieved": flops / gemm_ms / 1e9,
-                               "peak": FP32_ALU_TFLOPS, "unit": "TFLOP/s",
-                               "frac": flops / gemm_ms / 1e9 / FP32_ALU_TFLOPS,
-                               "peak_kind": "derived: 152 SMs x 128 FP32 lanes x 2 flop (FMA) x 2.07 GHz"}
+            pk, kind = tc_peak(sustained=True)
+            issued = 6 * flops / gemm_ms / 1e9
+            res["roofline"] = {"bound": "tensor", "kernel": "tc_c64_kernel (complex64: six bfloat16 MMAs per product)",
+                               "achieved": issued, "peak": pk, "unit": "TFLOP/s", "frac": issued / pk,
+                               "peak_kind": kind, "note": "achieved counts the six tensor-core products issued"}
         out[storage] = res
         op.close()
         torch.cuda.empty_cache()
@@ -747,7 +745,7 @@ def run_paper_full(args, dev):
             res[f"marchenko_nv{nv}"] = r
             del cut, fd, sol
             if storage == "c64":
-                break          # 20 points on complex64 run on the SIMT product (minutes); FP16 only
+                break          # 20 points: FP16 only
         op.close()
         out[storage] = res
     del x, yo, xo, fm_c64
