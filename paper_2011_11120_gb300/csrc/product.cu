@@ -793,7 +793,8 @@ bool gemv_fits(const mdc_plan* p, bool adjoint, int ncol, int cpv) {
     return ncol <= gemv_max_columns() && staged && red <= 200 * 1024;
 }
 
-// Default rule for column counts above the GEMV width: up to GEMV_GROUP_MAX_FWD (forward) or
+// Default rule for column counts above the GEMV width where no tensor-core product runs (operand buffers
+// missing): up to GEMV_GROUP_MAX_FWD (forward) or
 // GEMV_GROUP_MAX_ADJ (adjoint) columns the GEMV runs in passes over groups of 4, each streaming the
 // kernel near the HBM rate; above, the FP32 SIMT GEMM (128 x 32 tiles up to 32 columns).  The
 // crossover depends on the shape (measured on 8281^2, 3721 x 841 and 1681^2 complex64 kernels:
