@@ -64,3 +64,37 @@ def test_solver_epilogue_matches_oracle(nt, n, nv):
     for key, want in (("f_minus", res.x[0]), ("f_mplus", res.x[1]), ("g_minus", gm), ("g_plus", gp)):
         assert rel(out[key].cpu().numpy(), want) <= 1e-5, key
     assert np.allclose(out["resid"], res.resid, rtol=1e-5, atol=0)
+
+
+def chain_norm(d, nt, C):
+    """sqrt of the sum of squares of d [nt, C] as the inverse kernels form it: row rho of their tile holds the
+    sample t = (rho mod N2) N1 + rho / N2; rows of one column with equal rho mod TS are added up by float32
+    fused multiply-adds in ascending order, the chains and the columns in float64."""
+    N1, N2, CT = {64: (8, 8, 64), 128: (16, 8, 64), 256: (16, 16, 64), 512: (32, 16, 32), 1024: (32, 32, 16)}[nt]
+    TS = (4 if C % 4 == 0 else 1) * 256 // CT
+    rho = np.arange(nt)
+    rows = d[(rho % N2) * N1 + rho // N2].astype(np.float64)
+    ss = np.zeros((TS, C))
+    for m in range(nt // TS):
+        ss = (rows[m * TS:(m + 1) * TS] ** 2 + ss).astype(np.float32).astype(np.float64)
+    return np.sqrt(ss.sum())
+
+
+@pytest.mark.parametrize("nt", [64, 128, 256, 512, 1024])
+@pytest.mark.parametrize("n,nv", [(7, 3), (10, 1), (12, 3), (160, 4), (1601, 3)])
+def test_norm_does_not_depend_on_the_tile(nt, n, nv):
+    """The norm of a solve's data vector (few-column and full tiles) is the sum of the same chains.  Tolerance:
+    one chain in a thousand off by a rounding (2^-24), which float64 may take twice here."""
+    import paper_2011_11120_gb300 as m
+    nf = 6
+    rng, G = kernel(n, n, nf, nt + n)
+    cut = rng.integers(nt // 16, nt // 2, (n, nv)).astype(np.int32)
+    fd = torch.from_numpy(rng.standard_normal((nt, n, nv)).astype(np.float32)).cuda()
+    op = m.MDC(torch.from_numpy(G).cuda(), nt, 1.0, 1.0)
+    d = op.forward(fd).cpu().numpy().reshape(nt, n * nv)
+    resid = op.marchenko(torch.from_numpy(cut).cuda(), fd, 1)["resid"]
+    op.close()
+    t = np.arange(nt)
+    d[np.where(t < nt // 2, t, nt - t)[:, None] >= cut.reshape(1, -1)] = 0.0
+    want = chain_norm(d, nt, n * nv)
+    assert abs(resid[0] / want - 1.0) <= 1e-10
