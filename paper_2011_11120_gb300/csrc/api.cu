@@ -32,7 +32,6 @@ LaunchScope::~LaunchScope() {
     nvtxRangePop();
 }
 
-int ensure_scratch(mdc_plan* p, int ncols);
 
 }  // namespace mdc
 
@@ -244,7 +243,7 @@ extern "C" int mdc_create_weighted(mdc_handle* out, const void* G, const double*
     return create_plan(out, G, weights, nfmax, nr, ns, nt, dt, dr, storage, stream);
 }
 
-int mdc::ensure_scratch(mdc_plan* p, int ncols) {
+int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc) {
     if (ncols > p->nv_cap) {
         const size_t n = (size_t)p->nf * (size_t)(p->nr > p->ns ? p->nr : p->ns) * ncols;
         float2 *a = nullptr, *b = nullptr;
@@ -283,7 +282,7 @@ int mdc::ensure_scratch(mdc_plan* p, int ncols) {
     // complex64: the three-term operand of the tensor-core product.  It is three times the spectra, so
     // it is taken only where it leaves the caller three quarters of the free memory; without it the
     // products run on the GEMV / SIMT kernels.
-    if (p->storage == MDC_C64 && ncols >= C64_TC_MIN && ncols > p->tc_cap && ncols > p->tc_denied) {
+    if (c64_tc && p->storage == MDC_C64 && ncols >= C64_TC_MIN && ncols > p->tc_cap && ncols > p->tc_denied) {
         const size_t bytes = tc_c64_scratch_elems(p, ncols) * 2;
         size_t free_b = 0, total_b = 0;
         void* b = nullptr;

@@ -236,7 +236,7 @@ struct IrfftArgs {
     double* colsum;        // per-column sum of squares of out, or null
     const float2* tw;
     const int* active;
-    int vec4;              // set by the launcher: aligned 4-column output path
+    int vec4;              // set by the launcher: aligned 4-column output path (half-length transforms)
     // An LSQR step applied with the previous output v = out (before it is overwritten), same layout:
     //   xw_x <- xw_x + kx * xw_w,   xw_w <- ia * v + kw * xw_w     (kx, kw, ia: device doubles)
     // xw_w null: no step.  Needs the previous-output term and no time reversal.
@@ -268,9 +268,13 @@ inline int take_host_error(mdc_plan* p) {
 // Per-frequency products on the library layout.
 //   forward: Y[k][r][voff_o + j] = sum_s G[k][r][s] X[k][s][voff_i + j], j < ncol
 //   adjoint: X[k][s][voff_o + j] = sum_r conj(G[k][r][s]) Y[k][r][voff_i + j]
+// c64_tc: complex64 products may run on tensor cores (passes and deconvolution).  The Marchenko system's
+// stay on the float32 kernels: its Green's function g- = R f+ - f- can be a difference 50 to 450 times
+// smaller than its terms (a quarter of the inputs of 9 points on 1681 traces), and then shows any change of
+// rounding in the iterations at 1e-5 to 2e-4, although either product is equally far from 64 bits.
 void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i,
                     float2* out, int ldo, int voff_o, int ncol, cudaStream_t s,
-                    const int* active);
+                    const int* active, bool c64_tc = true);
 
 // Tensor-core products (tc_gemm.cu).
 bool tc_supported(const mdc_plan* p, int ncol);
@@ -308,5 +312,9 @@ inline bool storage_tc(int storage) {
 }
 
 void set_cuda_error(cudaError_t e);
+
+// Spectra and tensor-core operands for ncols columns (MDC_OK or MDC_ERR_OOM).  c64_tc: the complex64
+// tensor-core operand too, as launch_product.
+int ensure_scratch(mdc_plan* p, int ncols, bool c64_tc = true);
 
 }  // namespace mdc

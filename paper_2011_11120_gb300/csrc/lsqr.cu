@@ -25,7 +25,6 @@
 
 namespace mdc {
 
-int ensure_scratch(mdc_plan* p, int ncols);
 
 namespace {
 
@@ -133,11 +132,16 @@ struct Solver {
         launch_irfft(q, a, s);
     }
 
+    // specB <- product of specA over this system's first ncol columns (complex64 on the float32 kernels)
+    void product(mdc_plan* q, bool adjoint, int ncol, const int* active) {
+        launch_product(q, adjoint, q->specA, LD(), voff0, q->specB, LD(), voff0, ncol, s, active, false);
+    }
+
     // u-hat = d = [Theta R f_d+ ; 0] (kernel pr), column sums into csU; D1 keeps d for refinement.
     void data_pass(const float* fd) {
         const Coef zero = C1(0.f);
         rfft(pr, fd, nullptr, nullptr, C1(1.f), 0, 0, nullptr);
-        launch_product(pr, false, pr->specA, LD(), voff0, pr->specB, LD(), voff0, nv, s, nullptr);
+        product(pr, false, nv, nullptr);
         irfft(pr, 0, 0, U1(), C1(1.f), cut, nullptr, zero, zero, csU, 0, nullptr);
         cudaMemsetAsync(U2(), 0, B * sizeof(float), s);
         cudaMemsetAsync(csU + C, 0, C * sizeof(double), s);
@@ -156,7 +160,7 @@ struct Solver {
     void residual_pass(const float* x1, const float* x2) {
         rfft(pr, x2, nullptr, nullptr, C1(1.f), 0, 0, nullptr);
         rfft(pr, x1, nullptr, nullptr, C1(1.f), 1, nv, nullptr);
-        launch_product(pr, false, pr->specA, LD(), voff0, pr->specB, LD(), voff0, 2 * nv, s, nullptr);
+        product(pr, false, 2 * nv, nullptr);
         {
             LaunchScope ls(p, s, MDC_KC_SOLVER);
             copy_f<<<elementwise_grid(B), 256, 0, s>>>(B, D1(), U1());
@@ -171,7 +175,7 @@ struct Solver {
     void apply_MH(const int* active, Coef vprev) {
         rfft(p, U1(), nullptr, cut, CD(1.f, sc + S_INV_BETA), 0, 0, active);
         rfft(p, U2(), nullptr, cut, CD(1.f, sc + S_INV_BETA), 1, nv, active);
-        launch_product(p, true, p->specA, LD(), voff0, p->specB, LD(), voff0, 2 * nv, s, active);
+        product(p, true, 2 * nv, active);
         irfft(p, nv, 1, V1(), C1(-1.f), nullptr, U1(), CD(1.f, sc + S_INV_BETA), vprev, csV, 0, active, nullptr,
               nullptr, fuse_v ? nv : -1, nullptr, 1);
         irfft(p, 0, 0, V2(), C1(-1.f), nullptr, U2(), CD(1.f, sc + S_INV_BETA), vprev, csV + C, 0, active, nullptr,
@@ -252,10 +256,10 @@ struct Solver {
             const int* a = act0 + it;
             nvtxRangePushA("mdc lsqr iteration");
             iter_fwd_pre(a);
-            launch_product(p, false, p->specA, LD(), voff0, p->specB, LD(), voff0, 2 * nv, s, a);
+            product(p, false, 2 * nv, a);
             iter_fwd_post(a);
             iter_adj_pre(a);
-            launch_product(p, true, p->specA, LD(), voff0, p->specB, LD(), voff0, 2 * nv, s, a);
+            product(p, true, 2 * nv, a);
             iter_adj_post(it, niter, tol, act0, resid0, itp, x1, x2);
             nvtxRangePop();
         }
@@ -281,7 +285,7 @@ struct Solver {
         for (int k = 2; k <= niter; ++k) {
             rfft(p, x2, nullptr, nullptr, C1(1.f), 0, 0, nullptr);
             rfft(p, x1, nullptr, nullptr, C1(1.f), 1, nv, nullptr);
-            launch_product(p, false, p->specA, LD(), voff0, p->specB, LD(), voff0, 2 * nv, s, nullptr);
+            product(p, false, 2 * nv, nullptr);
             irfft(p, 0, 0, x1, C1(1.f), cut, D1(), C1(1.f), zero, nullptr, 0, nullptr);
             irfft(p, nv, 1, x2, C1(1.f), cut, nullptr, zero, zero, nullptr, 0, nullptr);
         }
@@ -297,7 +301,7 @@ struct Solver {
         }
         rfft(pr, fplus, nullptr, nullptr, C1(1.f), 0, 0, nullptr);
         rfft(pr, fm, nullptr, nullptr, C1(1.f), 1, nv, nullptr);
-        launch_product(pr, false, pr->specA, LD(), voff0, pr->specB, LD(), voff0, 2 * nv, s, nullptr);
+        product(pr, false, 2 * nv, nullptr);
         if (gm) irfft(pr, 0, 0, gm, C1(1.f), nullptr, fm, C1(-1.f), zero, nullptr, 0, nullptr);
         if (gp) irfft(pr, nv, 1, gp, C1(-1.f), nullptr, fplus, C1(1.f), zero, nullptr, 1, nullptr);
     }
@@ -371,8 +375,8 @@ int run_marchenko(mdc_plan* p, mdc_plan* pr, const int* cut, const float* fd, in
     // a frequency shard solves in lock step with the others only through its sum over shards
     if ((p->shard && !p->red_fn) || (pr->shard && !pr->red_fn)) return MDC_ERR_STATE;
     if (pr->k0 != p->k0 || pr->shard != p->shard) return MDC_ERR_ARG;
-    int st = ensure_scratch(p, 2 * nv);
-    if (st == MDC_OK && pr != p) st = ensure_scratch(pr, 2 * nv);
+    int st = ensure_scratch(p, 2 * nv, false);
+    if (st == MDC_OK && pr != p) st = ensure_scratch(pr, 2 * nv, false);
     if (st != MDC_OK) return st;
     const bool keep_data = nref > 0 || final_h != nullptr;
     Solver local;
@@ -507,7 +511,7 @@ extern "C" int marchenko_neumann(mdc_handle R, const int* window, const float* f
     if (R->nr != R->ns) return MDC_ERR_ARG;
     if (R->shard && !R->red_fn) return MDC_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
-    int st = mdc::ensure_scratch(R, 2 * nv);
+    int st = mdc::ensure_scratch(R, 2 * nv, false);
     if (st != MDC_OK) return st;
     mdc::Solver S;
     mdc::init_solver(S, R, R, window, nv, 1, 0, 0, s);
@@ -831,8 +835,8 @@ extern "C" int srv_create(mdc_server** out, mdc_handle R, mdc_handle R_ref, int6
     // one product path for every batch composition: a job's columns see the same arithmetic
     // alone or in a mix
     R->force_tc = (R->storage == MDC_C16F || R->storage == MDC_CBF16 || R->storage == MDC_CE4M3);
-    int st = ensure_scratch(R, max_cols);
-    if (st == MDC_OK && v->pr != R) st = ensure_scratch(v->pr, max_cols);
+    int st = ensure_scratch(R, max_cols, false);
+    if (st == MDC_OK && v->pr != R) st = ensure_scratch(v->pr, max_cols, false);
     if (st != MDC_OK) {
         delete v;
         return st;
@@ -912,10 +916,10 @@ extern "C" int srv_step(mdc_server* v, int* completed) {
             act[i] = j->S->act + j->aoff + j->it + 1;
             j->S->iter_fwd_pre(act[i]);
         }
-        launch_product(v->p, false, v->p->specA, L, 0, v->p->specB, L, 0, L, v->s, nullptr);
+        launch_product(v->p, false, v->p->specA, L, 0, v->p->specB, L, 0, L, v->s, nullptr, false);
         for (int i = 0; i < nrun; ++i) v->running[i]->S->iter_fwd_post(act[i]);
         for (int i = 0; i < nrun; ++i) v->running[i]->S->iter_adj_pre(act[i]);
-        launch_product(v->p, true, v->p->specA, L, 0, v->p->specB, L, 0, L, v->s, nullptr);
+        launch_product(v->p, true, v->p->specA, L, 0, v->p->specB, L, 0, L, v->s, nullptr, false);
         for (int i = 0; i < nrun; ++i) {
             ServeJob* j = v->running[i];
             const int niter = j->solve == 0 ? j->niter : v->niter_ref;

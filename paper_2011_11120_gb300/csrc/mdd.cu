@@ -18,7 +18,6 @@
 
 namespace mdc {
 
-int ensure_scratch(mdc_plan* p, int ncols);
 
 namespace {
 

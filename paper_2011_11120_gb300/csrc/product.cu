@@ -880,7 +880,7 @@ bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi
 
 void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i,
                     float2* out, int ldo, int voff_o, int ncol, cudaStream_t s,
-                    const int* active) {
+                    const int* active, bool c64_tc) {
     int path = PATH_AUTO, bn = 0;
     if (!p->force_tc) {
         // autotuned variant of the smallest tuned bucket holding ncol columns
@@ -904,7 +904,7 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
     }
     if (tc_wanted) ++p->tc_fallbacks;
     // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand buffers exist
-    if ((path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN)) && tc_c64_ready(p, ncol) &&
+    if (c64_tc && (path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN)) && tc_c64_ready(p, ncol) &&
         launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, true))
         return;
     LaunchScope ls(p, s, adjoint ? MDC_KC_PRODUCT_ADJ : MDC_KC_PRODUCT_FWD);
@@ -1002,7 +1002,6 @@ void launch_quantize(mdc_plan* p, const float2* G, const float* w, cudaStream_t 
 
 namespace mdc {
 
-int ensure_scratch(mdc_plan* p, int ncols);
 
 static std::string tune_key(const mdc_plan* p) {
     cudaDeviceProp prop{};

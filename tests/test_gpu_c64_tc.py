@@ -73,3 +73,29 @@ def test_c64_tensor_core_wait_limit():
     m.mdc_device_status(op.h)
     op.close()
     assert rel(yg, omdc.forward(G.astype(np.complex128), x, 0.004, 400.0)) <= TOL
+
+
+@pytest.mark.parametrize("nv", [3, 9])
+def test_marchenko_products_stay_in_float32(nv):
+    """A solve's complex64 products run on the float32 kernels, whether or not the handle holds the operand
+    that passes of as many columns use: the same bits either way."""
+    import paper_2011_11120_gb300 as m
+    nt, n, nf = 128, 70, 20
+    rng = np.random.default_rng(nv)
+    G = (rng.standard_normal((nf, n, n)) + 1j * rng.standard_normal((nf, n, n))) * (0.2 / np.sqrt(n))
+    cut = torch.from_numpy(rng.integers(nt // 16, nt // 2, (n, nv)).astype(np.int32)).cuda()
+    fd = torch.from_numpy(rng.standard_normal((nt, n, nv)).astype(np.float32)).cuda()
+    got = []
+    for reserve in (False, True):
+        op = m.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), nt, 1.0, 1.0)
+        if reserve:
+            m.mdc_reserve(op.h, 2 * nv)
+        m.mdc_timing(op.h, True)
+        out, neu = op.marchenko(cut, fd, 3), op.neumann(cut, fd, 3)
+        assert m.mdc_timing_read(op.h, "tc_prep")[1] == 0
+        op.forward(fd.repeat(1, 1, 2))
+        assert m.mdc_timing_read(op.h, "tc_prep")[1] == 1          # a pass of 2 nv columns does use it
+        got.append([t[k].cpu().numpy() for t in (out, neu) for k in ("f_minus", "f_mplus", "g_minus", "g_plus")])
+        op.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
