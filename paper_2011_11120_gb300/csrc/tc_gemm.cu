@@ -613,15 +613,16 @@ __global__ void __launch_bounds__(CVT ? TC_THREADS + TC_CVT_THREADS + 32 : TC_TH
 //
 // The leader (rank 0) owns the full barriers (both CTAs' loads report there) and issues the MMAs; their
 // commits release the stage and hand over the accumulator in both CTAs.  Both epilogues report the
-// accumulator empty to the leader.  Every wait is bounded as in tc_gemm_kernel; both CTAs always reach
-// the closing cluster barrier, before which the leader has seen all copies land and all MMAs complete.
+// accumulator empty to the leader.  Every wait is bounded as in tc_gemm_kernel.
+//
+// Leaving.  Each producer waits on the empty barriers of its own CTA, so after an expired wait one may have
+// issued up to PR_STAGES steps more than the other.  Both CTAs therefore meet at a cluster barrier once no
+// warp issues copies or MMAs any more; there the leader knows both step counts, settles the bytes that its
+// barriers still expect or were never told of, and waits for every copy of both CTAs.  No CTA leaves before
+// a second cluster barrier.
 constexpr int PR_BN = 256;
 constexpr int PR_STAGES = 6;
 constexpr uint32_t PR_A_BYTES = TC_BM * 128, PR_B_BYTES = (PR_BN / 2) * 128, PR_STAGE = PR_A_BYTES + PR_B_BYTES;
-
-// Bound on the leader's wait for each of the last copies: they land in microseconds, but the barrier
-// also counts the other CTA's, which may have given up.
-constexpr unsigned long long PR_DRAIN_NS = 20000000ull;
 
 constexpr size_t pair_smem_bytes() {
     // + alignment, barriers, two 128-float column-scale buffers, eight staging tiles
@@ -637,6 +638,10 @@ __device__ __forceinline__ uint32_t leader_addr(uint32_t addr) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
     return r;
+}
+// Bytes of the current phase that no copy will report.
+__device__ __forceinline__ void mbar_complete_tx(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -676,12 +681,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     const uint32_t raw = su32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
-    // full[S], empty[S], acc_full[2], acc_empty[2], drain, tmem slot; column scales 256 bytes on
+    // full[S], empty[S], acc_full[2], acc_empty[2], drain, tmem slot, step count of rank 1 (the leader's copy
+    // is used); column scales 256 bytes on
     uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + PR_STAGES * PR_STAGE);
     const uint32_t full0 = su32(bars), empty0 = full0 + 8 * PR_STAGES;
     const uint32_t accf0 = empty0 + 8 * PR_STAGES, acce0 = accf0 + 16, drain0 = acce0 + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * PR_STAGES + 5);
-    static_assert(2 * PR_STAGES + 6 <= 32, "barrier space");
+    uint32_t* peer_steps = reinterpret_cast<uint32_t*>(bars + 2 * PR_STAGES + 6);
+    static_assert(2 * PR_STAGES + 7 <= 32, "barrier space");
     float* sig_s = reinterpret_cast<float*>(bars + 32);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cta_rank();
@@ -721,6 +728,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
         n0 = (rem - mt * n_tiles_n) * PR_BN;
     };
 
+    uint32_t steps = 0;                              // thread 0: steps whose copies it issued
     if (warp == 0) {
         if (lane == 0) {
             long g = 0;
@@ -747,10 +755,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
                     tma_load_3d_pair(sb, &tmB, bar, kb * TC_BK, n0 + (int)rank * (PR_BN / 2), k);
                 }
             }
-            // both CTAs' copies have landed (they all report here) before either CTA can exit
-            if (rank == 0)
-                for (long q = g > PR_STAGES ? g - PR_STAGES : 0; q < g; ++q)
-                    mbar_wait(full0 + 8 * (int)(q % PR_STAGES), (uint32_t)(q / PR_STAGES) & 1, a.err, 42, PR_DRAIN_NS);
+            steps = (uint32_t)g;
+            if (rank == 1)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(leader_addr(su32(peer_steps))), "r"(steps)
+                             : "memory");
         }
     } else if (warp == 1) {
         if (rank == 0 && lane == 0) {
@@ -782,8 +790,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
                 umma_commit_pair(accf0 + 8 * buf);
             }
             // every MMA has completed before either CTA frees TMEM
-            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain0)
-                         : "memory");
+            umma_commit_pair(drain0);
             mbar_wait(drain0, 0, a.err, 45, TC_DRAIN_NS);
         }
     } else {
@@ -828,6 +835,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
         }
     }
     tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                          // no more copies and MMAs are issued; rank 1's count is here
+    if (threadIdx.x == 0) {
+        if (rank == 0) {
+            // a slot's barrier has completed every phase before that of the slot's last step: whoever issued
+            // that step had seen the MMAs of the one before, which waited for it
+            const uint32_t n1 = *peer_steps, last = steps > n1 ? steps : n1;
+            for (uint32_t q = last > PR_STAGES ? last - PR_STAGES : 0; q < last; ++q) {
+                const uint32_t bar = full0 + 8 * (q % PR_STAGES);
+                if (q >= steps) mbar_expect_tx(bar, PR_STAGE);              // rank 1's copies alone
+                else if (q >= n1) mbar_complete_tx(bar, PR_STAGE);          // the leader's copies alone
+                mbar_wait(bar, (q / PR_STAGES) & 1, a.err, 42, TC_DRAIN_NS);
+            }
+        } else {
+            mbar_wait(drain0, 0, a.err, 47, TC_DRAIN_NS);      // the leader's last commit has arrived here too
+        }
+    }
     __syncthreads();
     cluster_sync_all();                          // no CTA leaves while the other may signal or use it
     if (warp == 0) {

@@ -62,3 +62,33 @@ def test_pair_wait_limit():
     m.mdc_device_status(op.h)
     op.close()
     assert rel(yg, omdc.forward(dequantised(G, "c16f"), x, 0.004, 400.0)) <= 4 * FORMATS["c16f"][0]
+
+
+@pytest.mark.parametrize("nr,ns", [(300, 1100), (700, 2300)])
+def test_pair_leaves_nothing_behind(nr, ns):
+    """Limits around the time of a step, so that waits run out in some pairs and in either CTA of a pair, at any
+    step: every launch ends, its status is a timeout or none, and products launched right behind it on the
+    same SMs are right."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(nr, ns, 20, 100)
+    op = m.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), 64, 0.004, 400.0, storage="c16f")
+    xt, yt = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+    Gq = dequantised(G, "c16f")
+    want_y, want_x = omdc.forward(Gq, x, 0.004, 400.0), omdc.adjoint(Gq, y, 0.004, 400.0)
+    expired = 0
+    for us in (1, 2, 3, 5, 8, 12, 20, 30):
+        m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, us)
+        for _ in range(3):
+            op.forward(xt)
+            op.adjoint(yt)
+        m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, 0)
+        yg, xg = op.forward(xt).cpu().numpy(), op.adjoint(yt).cpu().numpy()
+        try:
+            m.mdc_device_status(op.h)
+        except m.MDCError as e:
+            assert e.status == -4
+            expired += 1
+        assert rel(yg, want_y) <= 4 * FORMATS["c16f"][0]
+        assert rel(xg, want_x) <= 4 * FORMATS["c16f"][0]
+    assert expired > 0
+    op.close()
