@@ -347,7 +347,9 @@ int srv_submit(mdc_server_handle s, const int* window_host, const float* fd_plus
                int niter, double tol, float* f_minus_host, float* f_mplus_host, float* g_minus_host,
                float* g_plus_host, int64_t* job_id);
 /* srv_step -- admit, advance every running job by one iteration, complete finished jobs
- * (their host outputs are written before return).  Blocking.  *completed = jobs completed. */
+ * (their host outputs are written before return).  Blocking.  *completed = jobs completed or failed.
+ * If a bounded device wait of R or R_ref ran out, every running job fails with MDC_ERR_TIMEOUT (from
+ * srv_poll); jobs submitted later are unaffected. */
 int srv_step(mdc_server_handle s, int* completed);
 /* srv_poll -- state (MDC_JOB_*), iterations, final residual ratio, latency (submit to
  * completion, s) and queueing delay (submit to admission, s); -1 where not yet known.

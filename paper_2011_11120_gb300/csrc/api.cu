@@ -438,7 +438,9 @@ extern "C" int mdc_device_status(mdc_handle h, void* stream) {
     if (v != 0) {
         MDC_CUDA_TRY(cudaMemsetAsync(h->err_flag, 0, sizeof(int), (cudaStream_t)stream));
         MDC_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
-        return mdc::device_flag_status(v);
+    } else {
+        v = h->err_seen;
     }
-    return MDC_OK;
+    h->err_seen = 0;
+    return mdc::device_flag_status(v);
 }

@@ -147,6 +147,7 @@ struct mdc_plan {
     int tc_cap = 0;
     int tc_denied = 0;          // complex64: columns whose operand did not fit (products run without it)
     int* err_flag = nullptr;    // device int: non-zero after a bounded device wait gave up
+    int err_seen = 0;           // a value of it that the server took (and cleared), for mdc_device_status
     unsigned long long wait_ns = 2000000000ull;   // bound on each tensor-core pipeline wait
     int64_t tc_fallbacks = 0;   // products the tensor-core rule chose that ran on another path
     bool force_tc = false;      // FP16/BF16: tensor-core products for every column count

@@ -472,6 +472,7 @@ int run_marchenko(mdc_plan* p, mdc_plan* pr, const int* cut, const float* fd, in
     }
     int err = 0;
     cudaMemcpy(&err, p->err_flag, sizeof(int), cudaMemcpyDeviceToHost);
+    if (!err && pr != p) cudaMemcpy(&err, pr->err_flag, sizeof(int), cudaMemcpyDeviceToHost);
     if (err) return mdc::device_flag_status(err);
     const int he = take_host_error(p), her = pr != p ? take_host_error(pr) : MDC_OK;
     if (he != MDC_OK) return he;
@@ -596,8 +597,8 @@ struct mdc_server {
     std::deque<ServeJob*> queue;
     std::vector<ServeJob*> running;
     std::unordered_map<int64_t, ServeJob*> jobs;
-    int* flags_h = nullptr;      // pinned
-    int flags_cap = 0;
+    int* flags_h = nullptr;      // pinned: a continue flag per running job, then the two handles' error flags
+    int flags_cap = 0;           // running jobs it holds
     bool keep_results = false;   // keep outputs given as NULL for srv_result
 };
 
@@ -785,6 +786,36 @@ int restore_job(mdc_server* v, ServeJob* j, const CkptJob& r, const unsigned cha
     return MDC_OK;
 }
 
+// The device error flags of the server's handles, into the pinned flags at position at, at + 1.
+void copy_error_flags(mdc_server* v, int at) {
+    cudaMemcpyAsync(v->flags_h + at, v->p->err_flag, sizeof(int), cudaMemcpyDeviceToHost, v->s);
+    cudaMemcpyAsync(v->flags_h + at + 1, v->pr->err_flag, sizeof(int), cudaMemcpyDeviceToHost, v->s);
+}
+
+// Status of the flags copied there (after a synchronisation).  A flag that was set is cleared, so that jobs
+// to come are judged by their own steps, and kept for mdc_device_status.
+int take_error_flags(mdc_server* v, int at) {
+    int st = MDC_OK;
+    mdc_plan* h[2] = {v->p, v->pr};
+    for (int i = 0; i < 2; ++i) {
+        const int e = v->flags_h[at + i];
+        if (!e) continue;
+        if (!h[i]->err_seen) h[i]->err_seen = e;
+        cudaMemsetAsync(h[i]->err_flag, 0, sizeof(int), v->s);
+        if (st == MDC_OK) st = device_flag_status(e);
+    }
+    return st;
+}
+
+void retire_job(mdc_server* v, ServeJob* j, int status) {
+    j->t_done = now_s();
+    j->state = status == MDC_OK ? JOB_DONE : JOB_FAILED;
+    if (status != MDC_OK) j->status = status;
+    v->used -= j->bytes;
+    v->cols -= 2 * j->nv;
+    free_job_device(v, j);
+}
+
 // Complete a finished job: float32 residual check, Green's functions, results to the host.
 void finish_job(mdc_server* v, ServeJob* j) {
     Solver* S = j->S;
@@ -837,6 +868,13 @@ extern "C" int srv_create(mdc_server** out, mdc_handle R, mdc_handle R_ref, int6
     R->force_tc = (R->storage == MDC_C16F || R->storage == MDC_CBF16 || R->storage == MDC_CE4M3);
     int st = ensure_scratch(R, max_cols, false);
     if (st == MDC_OK && v->pr != R) st = ensure_scratch(v->pr, max_cols, false);
+    // error flags of earlier calls are mdc_device_status' to report, not its jobs'
+    for (mdc_plan* h : {v->p, v->pr}) {
+        int e = 0;
+        if (st == MDC_OK && cudaMemcpy(&e, h->err_flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = MDC_ERR_CUDA;
+        if (e && !h->err_seen) h->err_seen = e;
+        if (e) cudaMemset(h->err_flag, 0, sizeof(int));
+    }
     if (st != MDC_OK) {
         delete v;
         return st;
@@ -932,7 +970,7 @@ extern "C" int srv_step(mdc_server* v, int* completed) {
         if (v->flags_cap < nrun) {
             if (v->flags_h) cudaFreeHost(v->flags_h);
             v->flags_cap = nrun * 2;
-            if (cudaMallocHost((void**)&v->flags_h, v->flags_cap * sizeof(int)) != cudaSuccess) {
+            if (cudaMallocHost((void**)&v->flags_h, (v->flags_cap + 2) * sizeof(int)) != cudaSuccess) {
                 v->flags_h = nullptr;
                 v->flags_cap = 0;
                 return MDC_ERR_OOM;
@@ -943,10 +981,20 @@ extern "C" int srv_step(mdc_server* v, int* completed) {
             cudaMemcpyAsync(v->flags_h + i, j->S->act + j->aoff + j->it + 1, sizeof(int), cudaMemcpyDeviceToHost,
                             v->s);
         }
+        copy_error_flags(v, nrun);
         cudaError_t e = cudaStreamSynchronize(v->s);
         if (e != cudaSuccess) {
             set_cuda_error(e);
             return MDC_ERR_CUDA;
+        }
+        // a wait that ran out, in this step's products or in the passes that started or refined a job since
+        // the last synchronisation, left spectra incomplete: every running job fails
+        const int bad_step = take_error_flags(v, nrun);
+        if (bad_step != MDC_OK) {
+            for (ServeJob* j : v->running) retire_job(v, j, bad_step);
+            v->running.clear();
+            if (completed) *completed = ndone + nrun;
+            return MDC_OK;
         }
         // 4. finished solves: refine or complete
         std::vector<ServeJob*> keep, fin;
@@ -981,25 +1029,28 @@ extern "C" int srv_step(mdc_server* v, int* completed) {
                 cudaMemcpyAsync(&res[q], fin[q]->S->xs + X_FINAL, sizeof(double), cudaMemcpyDeviceToHost, v->s);
                 cudaMemcpyAsync(&bad[q], fin[q]->S->sc + S_STATUS, sizeof(double), cudaMemcpyDeviceToHost, v->s);
             }
+            copy_error_flags(v, nrun);
             e = cudaStreamSynchronize(v->s);
             if (e != cudaSuccess) {
                 set_cuda_error(e);
                 return MDC_ERR_CUDA;
             }
+            const int bad_end = take_error_flags(v, nrun);
             for (size_t q = 0; q < fin.size(); ++q) {
                 ServeJob* j = fin[q];
                 int tot = 0;
                 for (int x : its[q]) tot += x;
                 j->iters = tot;
                 j->final_resid = res[q];
-                j->t_done = now_s();
                 // a non-finite alpha or beta retires this job alone: its batch mates' columns never mix with it
-                j->state = (bad[q] != 0.0 || !std::isfinite(res[q])) ? JOB_FAILED : JOB_DONE;
-                if (j->state == JOB_FAILED) j->status = MDC_ERR_NUMERIC;
-                v->used -= j->bytes;
-                v->cols -= 2 * j->nv;
-                free_job_device(v, j);
+                const bool numeric = bad[q] != 0.0 || !std::isfinite(res[q]);
+                retire_job(v, j, bad_end != MDC_OK ? bad_end : (numeric ? MDC_ERR_NUMERIC : MDC_OK));
                 ++ndone;
+            }
+            if (bad_end != MDC_OK) {             // it may have been a refinement pass of a job that goes on
+                for (ServeJob* j : keep) retire_job(v, j, bad_end);
+                ndone += (int)keep.size();
+                keep.clear();
             }
         }
         v->running.swap(keep);
