@@ -147,7 +147,10 @@ int mdc_forward(mdc_handle h, const float* x, float* y, int nv, unsigned flags, 
  */
 int mdc_adjoint(mdc_handle h, const float* y, float* x, int nv, unsigned flags, void* stream);
 
-/* mdc_reserve -- size the handle's scratch for up to nv_max columns per pass (blocking). */
+/* mdc_reserve -- size the handle's scratch for up to nv_max columns per pass (blocking).  With complex64
+ * storage and nv_max >= 5 that includes the operand of the tensor-core product, three times one spectrum of
+ * nv_max columns, if it is at most a quarter of the free memory (else the part of it that is, at least 64
+ * columns, or none; see MDC_OPT_C64_OPERAND_MB).  A call with more columns than reserved does the same. */
 int mdc_reserve(mdc_handle h, int nv_max);
 
 /*
@@ -225,7 +228,7 @@ int mdc_set_allreduce(mdc_handle h, mdc_allreduce_fn fn, void* ctx);
  * on tensor cores only if the handle's operand buffers were reserved beforehand
  * (mdc_reserve(h, nv), which allocates, so call it at set-up); otherwise the product
  * runs on the slower SIMT path (correct, and counted by mdc_tc_fallback_count).  The same holds
- * for complex64 storage from 5 columns on (not counted).
+ * for complex64 storage from 5 columns on.
  * Arguments, layout, ownership and errors are otherwise those of mdc_forward.
  */
 #define MDC_STATIC_SCRATCH_COMPLEX (1 << 21)
@@ -449,10 +452,17 @@ int mdc_autotune_choice(mdc_handle h, int adjoint, int ncol, int* path, int* bn)
  * memory and exit; the product's output is then incomplete.  Negative values: MDC_ERR_ARG.
  * (Failure detection: a limit the pipeline cannot meet exercises that path.) */
 #define MDC_OPT_WAIT_LIMIT_US 2
+/* MDC_OPT_C64_OPERAND_MB (value >= 0): largest operand, in MiB, that a complex64 handle takes for its
+ * tensor-core products (passes and deconvolution of 5 or more columns); 0 restores the default of a quarter
+ * of the memory that is free when it is taken.  Products of more columns than the operand holds run in
+ * slabs (the same result); with less than one tile (64 columns, or all of fewer) they run on the slower
+ * float32 kernels, counted by mdc_tc_fallback_count, and each further call tries again.  A larger operand
+ * that the handle holds is freed.  Negative values: MDC_ERR_ARG. */
+#define MDC_OPT_C64_OPERAND_MB 3
 int mdc_set_option(mdc_handle h, int option, int value);
 /* mdc_tc_fallback_count -- number of per-frequency products, since the handle was created, that
  * the tensor-core rule assigned to tensor cores (16-bit, split or E4M3 storage at 8 or more
- * columns, or an autotuned tensor-core choice) but that ran on the SIMT/GEMV path instead, because
+ * columns, complex64 passes and deconvolution at 5 or more, or an autotuned tensor-core choice) but that ran on the SIMT/GEMV path instead, because
  * the tensor-core operand buffers were not reserved for that many columns (mdc_reserve) or the
  * launch could not be set up.  Results are correct either way; the count exposes the slower
  * path.  -1 for a NULL handle.  Host-only. */

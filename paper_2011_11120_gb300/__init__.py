@@ -23,7 +23,7 @@ MDC_OK = 0
 MDC_C64, MDC_C16F, MDC_CBF16, MDC_CE4M3, MDC_C32S = 0, 1, 2, 3, 4
 STORAGE = {"c64": MDC_C64, "c16f": MDC_C16F, "cbf16": MDC_CBF16, "ce4m3": MDC_CE4M3, "c32s": MDC_C32S}
 MDC_CONJ_KERNEL = 0x1
-MDC_OPT_GRAPHS, MDC_OPT_WAIT_LIMIT_US = 1, 2
+MDC_OPT_GRAPHS, MDC_OPT_WAIT_LIMIT_US, MDC_OPT_C64_OPERAND_MB = 1, 2, 3
 KC_RFFT, KC_PRODUCT_FWD, KC_PRODUCT_ADJ, KC_IRFFT, KC_SOLVER, KC_TC_PREP = range(6)
 KERNEL_CLASSES = {"rfft": KC_RFFT, "product_fwd": KC_PRODUCT_FWD, "product_adj": KC_PRODUCT_ADJ,
                   "irfft": KC_IRFFT, "solver": KC_SOLVER, "tc_prep": KC_TC_PREP}

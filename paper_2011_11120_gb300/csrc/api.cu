@@ -243,8 +243,35 @@ extern "C" int mdc_create_weighted(mdc_handle* out, const void* G, const double*
     return create_plan(out, G, weights, nfmax, nr, ns, nt, dt, dr, storage, stream);
 }
 
-int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc) {
-    if (ncols > p->nv_cap) {
+// complex64: the three-term operand of the tensor-core product for up to ncols columns.  It is three times the
+// spectra, so it is taken only where it leaves the caller three quarters of the free memory, else for as
+// many columns as that allows (the products then go in slabs, with the same bits) or, where not even one
+// column tile fits, not at all: the products run on the GEMV / SIMT kernels, are counted as fallbacks, and
+// the next call tries again.
+static void c64_operand(mdc_plan* p, int ncols, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    size_t free_b = 0, total_b = 0;
+    if (ncols <= p->tc_cap || cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    const size_t bound = p->c64_limit ? (size_t)p->c64_limit : free_b / 4, col = tc_c64_scratch_elems(p, 1) * 2;
+    const int cols = bound / col < (size_t)ncols ? (int)(bound / col) : ncols;
+    void* b = nullptr;
+    if (cols <= p->tc_cap || cols < (ncols < C64_TILE_COLS ? ncols : C64_TILE_COLS)) return;
+    if (cudaMalloc(&b, col * cols) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    cudaFree(p->tcB);
+    p->tcB = b;
+    p->tc_cap = cols;
+}
+
+int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc, cudaStream_t s) {
+    const bool grown = ncols > p->nv_cap;
+    if (grown) {
         const size_t n = (size_t)p->nf * (size_t)(p->nr > p->ns ? p->nr : p->ns) * ncols;
         float2 *a = nullptr, *b = nullptr;
         cudaError_t e = cudaMalloc(&a, n * sizeof(float2));
@@ -279,36 +306,22 @@ int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc) {
         p->tcSigma = sg;
         p->tc_cap = ncols;
     }
-    // complex64: the three-term operand of the tensor-core product.  It is three times the spectra, so
-    // it is taken only where it leaves the caller three quarters of the free memory; without it the
-    // products run on the GEMV / SIMT kernels.
-    if (c64_tc && p->storage == MDC_C64 && ncols >= C64_TC_MIN && ncols > p->tc_cap && ncols > p->tc_denied) {
-        const size_t bytes = tc_c64_scratch_elems(p, ncols) * 2;
-        size_t free_b = 0, total_b = 0;
-        void* b = nullptr;
-        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4 &&
-            cudaMalloc(&b, bytes) == cudaSuccess) {
-            cudaFree(p->tcB);
-            p->tcB = b;
-            p->tc_cap = ncols;
-        } else {
-            cudaGetLastError();
-            p->tc_denied = ncols;
-        }
-    }
+    if (c64_tc && p->storage == MDC_C64 && ncols >= C64_TC_MIN && (grown || !tc_c64_ready(p, ncols))) c64_operand(p, ncols, s);
     return MDC_OK;
 }
 
 extern "C" int mdc_reserve(mdc_handle h, int nv_max) {
     if (!h || nv_max < 1) return MDC_ERR_ARG;
-    return ensure_scratch(h, nv_max);
+    const int st = ensure_scratch(h, nv_max);
+    if (st == MDC_OK && h->storage == MDC_C64 && nv_max >= C64_TC_MIN) c64_operand(h, nv_max, nullptr);
+    return st;
 }
 
 // One MDC pass: rFFT of `in` (S_in spatial points), per-frequency product, irFFT to `out`.
 static int mdc_pass(mdc_plan* p, bool adjoint, const float* in, float* outp, int nv, unsigned flags,
                     cudaStream_t s) {
     if (!in || !outp || nv < 1) return MDC_ERR_ARG;
-    int st = ensure_scratch(p, nv);
+    int st = ensure_scratch(p, nv, true, s);
     if (st != MDC_OK) return st;
     const int S_in = adjoint ? p->nr : p->ns;
     const int S_out = adjoint ? p->ns : p->nr;
@@ -422,6 +435,15 @@ extern "C" int mdc_set_option(mdc_handle h, int option, int value) {
         case MDC_OPT_WAIT_LIMIT_US:
             if (value < 0) return MDC_ERR_ARG;
             h->wait_ns = value == 0 ? 2000000000ull : (unsigned long long)value * 1000ull;
+            return MDC_OK;
+        case MDC_OPT_C64_OPERAND_MB:
+            if (value < 0) return MDC_ERR_ARG;
+            h->c64_limit = (int64_t)value << 20;
+            if (h->storage == MDC_C64 && value && (int64_t)(tc_c64_scratch_elems(h, 1) * 2 * h->tc_cap) > h->c64_limit) {
+                cudaFree(h->tcB);                // (waits for the products that use it)
+                h->tcB = nullptr;
+                h->tc_cap = 0;
+            }
             return MDC_OK;
         default:
             return MDC_ERR_ARG;

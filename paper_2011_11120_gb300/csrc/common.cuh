@@ -144,8 +144,8 @@ struct mdc_plan {
     // tensor-core path (FP16/BF16 storage): prepared B operand and its column scales
     void* tcB = nullptr;        // [nf][rows_pad][max(2*ldg, nr8)] 16-bit; complex64: three planes [nf][2 ncol][..]
     float* tcSigma = nullptr;   // [nf][tc_cap] (null for complex64)
-    int tc_cap = 0;
-    int tc_denied = 0;          // complex64: columns whose operand did not fit (products run without it)
+    int tc_cap = 0;             // columns they hold (complex64: wider products go in slabs of whole column tiles)
+    int64_t c64_limit = 0;      // bound on the complex64 operand in bytes (0: a quarter of the free memory)
     int* err_flag = nullptr;    // device int: non-zero after a bounded device wait gave up
     int err_seen = 0;           // a value of it that the server took (and cleared), for mdc_device_status
     unsigned long long wait_ns = 2000000000ull;   // bound on each tensor-core pipeline wait
@@ -293,7 +293,8 @@ size_t tc_scratch_elems(const mdc_plan* p, int ncol);
 // 1681^2 x 150, 10 / 16 and 8 / 14 us on 81^2 x 40; of 5 columns, GEMV in two groups / tensor cores:
 // 1.43 / 0.65 and 1.04 / 0.65 ms, 20 / 16 and 12 / 14 us.
 constexpr int C64_TC_MIN = 5;
-bool tc_c64_ready(const mdc_plan* p, int ncol);        // operand buffers exist for ncol columns
+constexpr int C64_TILE_COLS = 64;                      // columns of the widest tile: an operand of as many serves any product
+bool tc_c64_ready(const mdc_plan* p, int ncol);        // the operand holds ncol columns, or a tile of them
 size_t tc_c64_scratch_elems(const mdc_plan* p, int ncol);
 bool launch_tc_c64(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out, int ldo,
                    int voff_o, int ncol, cudaStream_t s, const int* active, bool scoped);
@@ -315,7 +316,7 @@ inline bool storage_tc(int storage) {
 void set_cuda_error(cudaError_t e);
 
 // Spectra and tensor-core operands for ncols columns (MDC_OK or MDC_ERR_OOM).  c64_tc: the complex64
-// tensor-core operand too, as launch_product.
-int ensure_scratch(mdc_plan* p, int ncols, bool c64_tc = true);
+// tensor-core operand too, as launch_product.  s: the calling stream (nothing is tried while it is captured).
+int ensure_scratch(mdc_plan* p, int ncols, bool c64_tc = true, cudaStream_t s = nullptr);
 
 }  // namespace mdc

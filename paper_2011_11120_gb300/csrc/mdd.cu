@@ -173,7 +173,7 @@ extern "C" int mdd_lsqr(mdc_handle Gplus, const float* g_minus, int nv, int nite
     mdc_plan* p = Gplus;
     if (p->shard && !p->red_fn) return MDC_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
-    int st = ensure_scratch(p, nv);
+    int st = ensure_scratch(p, nv, true, s);
     if (st != MDC_OK) return st;
     MddSolver S;
     S.p = p;

@@ -902,11 +902,13 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
             return;
         path = PATH_AUTO;
     }
-    if (tc_wanted) ++p->tc_fallbacks;
-    // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand buffers exist
-    if (c64_tc && (path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN)) && tc_c64_ready(p, ncol) &&
+    // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand exists
+    const bool c64_wanted =
+        c64_tc && p->storage == MDC_C64 && (path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN));
+    if (c64_wanted && tc_c64_ready(p, ncol) &&
         launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, true))
         return;
+    if (tc_wanted || c64_wanted) ++p->tc_fallbacks;
     LaunchScope ls(p, s, adjoint ? MDC_KC_PRODUCT_ADJ : MDC_KC_PRODUCT_FWD);
     if (!product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, path))
         product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, PATH_AUTO);

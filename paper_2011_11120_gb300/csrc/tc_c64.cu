@@ -578,14 +578,16 @@ size_t tc_c64_scratch_elems(const mdc_plan* p, int ncol) {
 }
 
 bool tc_c64_ready(const mdc_plan* p, int ncol) {
-    return p->storage == MDC_C64 && p->tcB != nullptr && ncol <= p->tc_cap && encode_fn() != nullptr;
+    return p->storage == MDC_C64 && p->tcB != nullptr && (ncol < C64_TILE_COLS ? ncol : C64_TILE_COLS) <= p->tc_cap &&
+           encode_fn() != nullptr;
 }
 
-bool launch_tc_c64(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out, int ldo,
-                   int voff_o, int ncol, cudaStream_t s, const int* active, bool scoped) {
+namespace {
+// Columns [voff, voff + ncol) with column tiles of bn real columns.
+bool c64_slab(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out, int ldo, int voff_o,
+              int ncol, int bn, cudaStream_t s, const int* active, bool scoped) {
     const int rows = adjoint ? p->nr : p->ns;                  // reduction rows of the spectra
     const int pitch = c64_pitch(p, adjoint);
-    const int bn = c64_bn(2 * ncol);
     const uint64_t kp = 2 * (uint64_t)p->ldg;
     auto enc = encode_fn();
     if (!enc) return false;
@@ -645,6 +647,20 @@ bool launch_tc_c64(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vof
         MDC_C64_CASE(128)
     }
 #undef MDC_C64_CASE
+    return true;
+}
+}  // namespace
+
+// An operand of fewer columns than the product's takes it slab by slab, each of whole column tiles, so the
+// sums are the same.
+bool launch_tc_c64(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i, float2* out, int ldo,
+                   int voff_o, int ncol, cudaStream_t s, const int* active, bool scoped) {
+    const int bn = c64_bn(2 * ncol), tile = bn / 2;
+    const int slab = ncol <= p->tc_cap ? ncol : p->tc_cap / tile * tile;
+    for (int c = 0; c < ncol; c += slab)
+        if (!c64_slab(p, adjoint, in, ldi, voff_i + c, out, ldo, voff_o + c, ncol - c < slab ? ncol - c : slab, bn, s,
+                      active, scoped))
+            return false;
     return true;
 }
 

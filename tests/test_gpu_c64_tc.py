@@ -99,3 +99,53 @@ def test_marchenko_products_stay_in_float32(nv):
         op.close()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+def test_operand_limit():
+    """A smaller operand takes wide products in slabs with the same bits; none at all sends them to the float32
+    kernels, counted, until a call finds room again."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(333, 700, 8, 200)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    xt, yt = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+
+    def both():
+        m.mdc_timing(op.h, True)
+        out = op.forward(xt).cpu().numpy(), op.adjoint(yt).cpu().numpy()
+        return out, m.mdc_timing_read(op.h, "tc_prep")[1], m.mdc_tc_fallback_count(op.h)
+
+    full, preps, count = both()
+    assert (preps, count) == (2, 0)
+    m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, 9)           # 69 of 200 columns: slabs of a 64-column tile
+    slabs, preps, count = both()
+    assert (preps, count) == (8, 0)
+    m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, 1)
+    none, preps, count = both()
+    assert (preps, count) == (0, 2)
+    m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, 0)
+    again, preps, count = both()
+    assert (preps, count) == (2, 2)
+    m.mdc_device_status(op.h)
+    op.close()
+    G = G.astype(np.complex128)
+    want = omdc.forward(G, x, 0.004, 400.0), omdc.adjoint(G, y, 0.004, 400.0)
+    for f, s, n, a, w in zip(full, slabs, none, again, want):
+        assert np.array_equal(f, s) and np.array_equal(f, a)
+        assert rel(f, w) <= TOL and rel(n, w) <= TOL
+
+
+@pytest.mark.parametrize("ncol", [20, 40])
+def test_float32_gemm_matches_oracle(ncol):
+    """The SIMT GEMM's narrow and wide tiles, which products without the operand run on, in both directions."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(131, 497, 9, ncol)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, 1)           # the operand takes 110 KB a column
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    used = m.mdc_tc_fallback_count(op.h)
+    op.close()
+    G = G.astype(np.complex128)
+    assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
+    assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
+    assert used == 2
