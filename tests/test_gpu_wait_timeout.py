@@ -82,10 +82,11 @@ def solve_problem(n, nf, nv, nt=64):
 
 
 def expire(m, op, nv):
-    """Run op's forward products under a limit they cannot meet; the device flag stays set."""
+    """Run op's forward products (a complex64 kernel far larger than L2, whose tiles take some microseconds to
+    load) under a limit they cannot meet; the device flag stays set."""
     x = torch.randn((op.nt, op.ns, nv), device="cuda")
     m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, 1)
-    for _ in range(20):
+    for _ in range(40):
         op.forward(x)
     m.mdc_set_option(op.h, m.MDC_OPT_WAIT_LIMIT_US, 0)
 
@@ -94,7 +95,7 @@ def test_timeout_on_the_reference_handle_is_reported():
     """The residual passes and Green's functions of a refined solve run on R_ref, whose device flag is the
     call's error as much as R's."""
     import paper_2011_11120_gb300 as m
-    G, cut, fd = solve_problem(1100, 20, 8)
+    G, cut, fd = solve_problem(1100, 30, 8)
     op = m.MDC(G, 64, 1.0, 1.0, storage="c16f")
     ref = m.MDC(G, 64, 1.0, 1.0, storage="c64")
     try:
@@ -115,7 +116,7 @@ def test_timeout_on_the_reference_handle_is_reported():
 def test_timeout_fails_the_running_jobs(which):
     import paper_2011_11120_gb300 as m
     nt, n, nv = 64, 4096, 8
-    G, cut, fd = solve_problem(n, 3, nv, nt)
+    G, cut, fd = solve_problem(n, 8, nv, nt)
     op = m.MDC(G, nt, 1.0, 1.0, storage="c16f")
     ref = m.MDC(G, nt, 1.0, 1.0, storage="c64")
     want = op.marchenko_refined(ref, cut, fd, 3, nrefine=0, niter_refine=1)
