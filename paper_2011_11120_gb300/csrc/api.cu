@@ -414,7 +414,7 @@ extern "C" int mdc_autotune_choice(mdc_handle h, int adjoint, int ncol, int* pat
     *bn = 0;
     for (const ProductChoice& c : h->tune[adjoint ? 1 : 0])
         if (ncol <= c.ncol) {
-            *path = c.path;
+            *path = c.path == PATH_C64_TC ? PATH_SIMT : c.path;
             *bn = c.bn;
             break;
         }

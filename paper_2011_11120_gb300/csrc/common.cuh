@@ -98,8 +98,9 @@ constexpr int G_PITCH_ALIGN = 64;
 struct EventPair { cudaEvent_t a, b; };
 
 // Product variant chosen by the autotuner for column counts up to `ncol`.
-// PATH_GEMV_GROUPS: GEMV passes over groups of up to 4 columns (one kernel read per group)
-enum ProductPath { PATH_AUTO = 0, PATH_GEMV = 1, PATH_SIMT = 2, PATH_TC = 3, PATH_GEMV_GROUPS = 4 };
+// PATH_GEMV_GROUPS: GEMV passes over groups of up to 4 columns (one kernel read per group); PATH_C64_TC: the
+// complex64 tensor-core GEMM (mdc_autotune_choice reports it as a float32 GEMM, 2)
+enum ProductPath { PATH_AUTO = 0, PATH_GEMV = 1, PATH_SIMT = 2, PATH_TC = 3, PATH_GEMV_GROUPS = 4, PATH_C64_TC = 5 };
 struct ProductChoice {
     int ncol;
     int path;
@@ -152,7 +153,9 @@ struct mdc_plan {
     int64_t tc_fallbacks = 0;   // products the tensor-core rule chose that ran on another path
     bool force_tc = false;      // FP16/BF16: tensor-core products for every column count
     bool graphs = false;        // capture repeated solves into CUDA graphs (mdc_set_option)
-    std::vector<mdc::ProductChoice> tune[2];   // autotuned variants [forward, adjoint], ascending ncol
+    // autotuned variants [forward, adjoint], ascending ncol; then, for complex64, those of the products that
+    // stay on the float32 kernels (launch_product with c64_tc false)
+    std::vector<mdc::ProductChoice> tune[4];
     std::vector<void*> graph_cache;   // solver workspaces with their instantiated graphs
     cudaStream_t graph_stream = nullptr;   // private stream for capture and replay
     cudaEvent_t graph_ev[2] = {nullptr, nullptr};

@@ -873,8 +873,9 @@ bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi
     if (path == PATH_TC)
         return storage_tc(p->storage) && p->tcB && ncol <= p->tc_cap &&
                launch_tc_product(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, bn);
-    if (path == PATH_SIMT && tc_c64_ready(p, ncol))
-        return launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, false);
+    if (path == PATH_C64_TC)
+        return tc_c64_ready(p, ncol) &&
+               launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, false);
     return product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, path);
 }
 
@@ -884,7 +885,8 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
     int path = PATH_AUTO, bn = 0;
     if (!p->force_tc) {
         // autotuned variant of the smallest tuned bucket holding ncol columns
-        for (const ProductChoice& c : p->tune[adjoint ? 1 : 0])
+        const int table = (p->storage == MDC_C64 && !c64_tc ? 2 : 0) + (adjoint ? 1 : 0);
+        for (const ProductChoice& c : p->tune[table])
             if (ncol <= c.ncol) {
                 path = c.path;
                 bn = c.bn;
@@ -904,7 +906,8 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
     }
     // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand exists
     const bool c64_wanted =
-        c64_tc && p->storage == MDC_C64 && (path == PATH_SIMT || (path == PATH_AUTO && ncol >= C64_TC_MIN));
+        c64_tc && p->storage == MDC_C64 && (path == PATH_C64_TC || (path == PATH_AUTO && ncol >= C64_TC_MIN));
+    if (path == PATH_C64_TC) path = PATH_AUTO;
     if (c64_wanted && tc_c64_ready(p, ncol) &&
         launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, true))
         return;
@@ -992,11 +995,13 @@ void launch_quantize(mdc_plan* p, const float2* G, const float* w, cudaStream_t 
 
 // ------------------------------------------------------------------ autotuner
 // For each direction and each column-count bucket (1, 2, 4, ..., up to ncol_max) time every
-// variant that can run -- GEMV (<= 4 columns), SIMT GEMM, and for 16-bit storage the tensor-core
-// GEMM with column tiles of 32, 64, 128 and 256 -- on the handle's own spectra with CUDA events
-// (one warm-up, median of three), and keep the fastest.  The table maps ncol to the variant of
-// the smallest bucket >= ncol.  With MDC_AUTOTUNE_CACHE set, tables are read from / appended to
-// that file (one JSON object per line) keyed by device name, shape and storage.
+// variant that can run -- GEMV (<= 4 columns), SIMT GEMM, for 16-bit storage the tensor-core
+// GEMM with column tiles of 32, 64, 128 and 256, for complex64 its own tensor-core GEMM -- on the handle's
+// own spectra with CUDA events (one warm-up, median of three), and keep the fastest (for complex64 the
+// fastest float32 kernel too, for the products that stay on those).  The table maps ncol to the variant of
+// the smallest bucket >= ncol.  With MDC_AUTOTUNE_CACHE set, tables are read from / appended to that file (one
+// JSON object per line) keyed by device name, shape, storage, the version of the kernel set and, for
+// complex64, whether the handle holds the tensor-core operand.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1005,14 +1010,17 @@ void launch_quantize(mdc_plan* p, const float2* G, const float* w, cudaStream_t 
 namespace mdc {
 
 
-static std::string tune_key(const mdc_plan* p) {
+// Raised when kernels or rules change so that older measurements no longer tell which variant is fastest.
+constexpr int TUNE_VERSION = 2;
+
+static std::string tune_key(const mdc_plan* p, int ncol_max) {
     cudaDeviceProp prop{};
     int dev = 0;
     cudaGetDevice(&dev);
     cudaGetDeviceProperties(&prop, dev);
     char buf[512];
-    snprintf(buf, sizeof(buf), "%s|nf=%d|nr=%d|ns=%d|nt=%d|storage=%d", prop.name, p->nf, p->nr, p->ns, p->nt,
-             p->storage);
+    snprintf(buf, sizeof(buf), "%s|nf=%d|nr=%d|ns=%d|nt=%d|storage=%d|v=%d%s", prop.name, p->nf, p->nr, p->ns, p->nt,
+             p->storage, TUNE_VERSION, p->storage != MDC_C64 ? "" : (tc_c64_ready(p, ncol_max) ? "|tc=1" : "|tc=0"));
     for (char* c = buf; *c; ++c)
         if (*c == '"' || *c == '\\') *c = '_';
     return buf;
@@ -1034,16 +1042,15 @@ static bool tune_load(mdc_plan* p, const std::string& key, int ncol_max) {
         q = strstr(line, "\"choices\": [");
         if (!q) continue;
         q += 12;
-        std::vector<ProductChoice> t[2];
+        std::vector<ProductChoice> t[4];
         int d, n, pa, bn, used;
-        while (sscanf(q, " [%d, %d, %d, %d]%n", &d, &n, &pa, &bn, &used) == 4 && (d == 0 || d == 1)) {
+        while (sscanf(q, " [%d, %d, %d, %d]%n", &d, &n, &pa, &bn, &used) == 4 && d >= 0 && d < 4) {
             t[d].push_back(ProductChoice{n, pa, bn});
             q += used;
             while (*q == ',' || *q == ' ') ++q;
         }
-        if (!t[0].empty() && !t[1].empty()) {
-            p->tune[0] = t[0];
-            p->tune[1] = t[1];
+        if (!t[0].empty() && !t[1].empty() && (p->storage != MDC_C64 || (!t[2].empty() && !t[3].empty()))) {
+            for (int i = 0; i < 4; ++i) p->tune[i] = t[i];
             found = true;
         }
     }
@@ -1058,7 +1065,7 @@ static void tune_store(const mdc_plan* p, const std::string& key, int ncol_max) 
     if (!f) return;
     fprintf(f, "{\"key\": \"%s\", \"ncol_max\": %d, \"choices\": [", key.c_str(), ncol_max);
     bool first = true;
-    for (int d = 0; d < 2; ++d)
+    for (int d = 0; d < 4; ++d)
         for (const ProductChoice& c : p->tune[d]) {
             fprintf(f, "%s[%d, %d, %d, %d]", first ? "" : ", ", d, c.ncol, c.path, c.bn);
             first = false;
@@ -1068,17 +1075,16 @@ static void tune_store(const mdc_plan* p, const std::string& key, int ncol_max) 
 }
 
 int autotune(mdc_plan* p, int ncol_max, cudaStream_t s) {
-    const std::string key = tune_key(p);
-    if (tune_load(p, key, ncol_max)) return MDC_OK;
     int st = ensure_scratch(p, ncol_max);
     if (st != MDC_OK) return st;
+    const std::string key = tune_key(p, ncol_max);
+    if (tune_load(p, key, ncol_max)) return MDC_OK;
     const size_t nspace = (size_t)(p->nr > p->ns ? p->nr : p->ns);
     cudaMemsetAsync(p->specA, 0, (size_t)p->nf * nspace * p->nv_cap * sizeof(float2), s);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    p->tune[0].clear();
-    p->tune[1].clear();
+    for (auto& t : p->tune) t.clear();
     for (int d = 0; d < 2; ++d) {
         const bool adj = d == 1;
         for (int n = 1;; n *= 2) {
@@ -1088,11 +1094,12 @@ int autotune(mdc_plan* p, int ncol_max, cudaStream_t s) {
             if (ncol <= gemv_max_columns()) cands.push_back({PATH_GEMV, 0});
             else if (ncol <= 64) cands.push_back({PATH_GEMV_GROUPS, 0});
             cands.push_back({PATH_SIMT, 0});
+            if (p->storage == MDC_C64) cands.push_back({PATH_C64_TC, 0});
             if (storage_tc(p->storage) && p->tcB)
                 for (int bn = 32; bn <= 256; bn *= 2)
                     if (bn / 2 <= 2 * ncol || bn == 32) cands.push_back({PATH_TC, bn});
-            float best = 1e30f;
-            ProductChoice pick{ncol, PATH_AUTO, 0};
+            float best = 1e30f, best32 = 1e30f;
+            ProductChoice pick{ncol, PATH_AUTO, 0}, pick32 = pick;      // of all, of the float32 kernels
             for (const Cand& c : cands) {
                 if (!launch_product_variant(p, adj, p->specA, ncol, 0, p->specB, ncol, 0, ncol, s, c.path, c.bn))
                     continue;
@@ -1110,8 +1117,13 @@ int autotune(mdc_plan* p, int ncol_max, cudaStream_t s) {
                     best = med;
                     pick = ProductChoice{ncol, c.path, c.bn};
                 }
+                if (c.path != PATH_C64_TC && med < best32) {
+                    best32 = med;
+                    pick32 = ProductChoice{ncol, c.path, c.bn};
+                }
             }
             p->tune[d].push_back(pick);
+            if (p->storage == MDC_C64) p->tune[2 + d].push_back(pick32);
             if (ncol >= ncol_max) break;
         }
     }
@@ -1120,8 +1132,7 @@ int autotune(mdc_plan* p, int ncol_max, cudaStream_t s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_cuda_error(e);
-        p->tune[0].clear();
-        p->tune[1].clear();
+        for (auto& t : p->tune) t.clear();
         return MDC_ERR_CUDA;
     }
     tune_store(p, key, ncol_max);

@@ -53,3 +53,37 @@ def test_autotune_choices_and_parity(tmp_path, storage):
         op2.close()
     finally:
         del os.environ["MDC_AUTOTUNE_CACHE"]
+
+
+def test_complex64_tables_tell_the_gemms_apart(tmp_path):
+    """Wide complex64 products of a tuned handle take the tensor-core GEMM, solves the float32 kernels; a handle
+    without the operand has a table of its own, and tables of earlier kernel sets are not read."""
+    import paper_2011_11120_gb300 as m
+    cache = tmp_path / "tune.jsonl"
+    os.environ["MDC_AUTOTUNE_CACHE"] = str(cache)
+    try:
+        rng = np.random.default_rng(4)
+        nt, nf, n, nv = 128, 24, 400, 40
+        G = (rng.standard_normal((nf, n, n)) + 1j * rng.standard_normal((nf, n, n))) * (0.2 / np.sqrt(n))
+        Gt = torch.from_numpy(G.astype(np.complex64)).cuda()
+        x = torch.from_numpy(rng.standard_normal((nt, n, nv)).astype(np.float32)).cuda()
+        cut = torch.from_numpy(rng.integers(nt // 16, nt // 2, (n, nv)).astype(np.int32)).cuda()
+        old = '{"key": "%s|nf=%d|nr=%d|ns=%d|nt=%d|storage=0", "ncol_max": 80, "choices": [[0, 80, 4, 0], [1, 80, 4, 0]]}\n'
+        cache.write_text(old % (torch.cuda.get_device_name(0), nf, n, n, nt))
+        preps, outs = [], []
+        for limit in (0, 1):
+            op = m.MDC(Gt, nt, 1.0, 1.0)
+            m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, limit)
+            m.mdc_autotune(op.h, 2 * nv)
+            m.mdc_timing(op.h, True)
+            y = op.forward(x)
+            preps.append(m.mdc_timing_read(op.h, "tc_prep")[1])
+            outs.append(op.marchenko(cut, x, 2)["f_minus"].cpu().numpy())
+            assert m.mdc_timing_read(op.h, "tc_prep")[1] == preps[-1]
+            assert rel(y.cpu().numpy(), omdc.forward(G, x.cpu().numpy(), 1.0, 1.0)) <= 1e-6
+            op.close()
+        assert preps == [1, 0]
+        assert rel(outs[0], outs[1].astype(np.float64)) <= 1e-5
+        assert len(cache.read_text().strip().splitlines()) == 3
+    finally:
+        del os.environ["MDC_AUTOTUNE_CACHE"]
