@@ -243,6 +243,11 @@ extern "C" int mdc_create_weighted(mdc_handle* out, const void* G, const double*
     return create_plan(out, G, weights, nfmax, nr, ns, nt, dt, dr, storage, stream);
 }
 
+static int64_t next_scratch_id() {
+    static std::atomic<int64_t> n{0};
+    return ++n;
+}
+
 // complex64: the three-term operand of the tensor-core product for up to ncols columns.  It is three times the
 // spectra, so it is taken only where it leaves the caller three quarters of the free memory, else for as
 // many columns as that allows (the products then go in slabs, with the same bits) or, where not even one
@@ -267,6 +272,7 @@ static void c64_operand(mdc_plan* p, int ncols, cudaStream_t s) {
     cudaFree(p->tcB);
     p->tcB = b;
     p->tc_cap = cols;
+    p->scratch_id = next_scratch_id();
 }
 
 int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc, cudaStream_t s) {
@@ -287,6 +293,7 @@ int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc, cudaStream_t s) {
         p->specA = a;
         p->specB = b;
         p->nv_cap = ncols;
+        p->scratch_id = next_scratch_id();
     }
     // tensor-core operand for the FP16/BF16/E4M3 copies (used from 8 columns on)
     if (storage_tc(p->storage) && ncols > p->tc_cap) {
@@ -305,6 +312,7 @@ int mdc::ensure_scratch(mdc_plan* p, int ncols, bool c64_tc, cudaStream_t s) {
         p->tcB = b;
         p->tcSigma = sg;
         p->tc_cap = ncols;
+        p->scratch_id = next_scratch_id();
     }
     if (c64_tc && p->storage == MDC_C64 && ncols >= C64_TC_MIN && (grown || !tc_c64_ready(p, ncols))) c64_operand(p, ncols, s);
     return MDC_OK;

@@ -140,6 +140,7 @@ struct mdc_plan {
                                 // conjugate (half-length transforms), from host float64
     // scratch spectra, sized for nv_cap columns
     int nv_cap = 0;
+    int64_t scratch_id = 0;     // changes whenever spectra or operands move (unique over all handles)
     float2* specA = nullptr;    // [nf][max(nr,ns)][nv_cap]
     float2* specB = nullptr;
     // tensor-core path (FP16/BF16 storage): prepared B operand and its column scales

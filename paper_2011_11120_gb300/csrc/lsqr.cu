@@ -310,6 +310,7 @@ struct Solver {
 struct GraphEntry {
     // key
     mdc_plan* pr;
+    int64_t scratch[2];        // scratch_id of both handles: the graph holds pointers into their scratch
     const int* cut;
     const float* fd;
     float* out[4];
@@ -397,6 +398,14 @@ int run_marchenko(mdc_plan* p, mdc_plan* pr, const int* cut, const float* fd, in
         s = p->graph_stream;
         cudaEventRecord(p->graph_ev[0], caller);
         cudaStreamWaitEvent(s, p->graph_ev[0], 0);
+        // solves captured before a wider call moved the scratch go (a destroyed and re-created pr has another id)
+        for (size_t i = p->graph_cache.size(); i-- > 0;) {
+            GraphEntry* g = static_cast<GraphEntry*>(p->graph_cache[i]);
+            if (g->scratch[0] == p->scratch_id && (g->pr != pr || g->scratch[1] == pr->scratch_id)) continue;
+            cudaStreamSynchronize(s);
+            free_graph_entry(g);
+            p->graph_cache.erase(p->graph_cache.begin() + i);
+        }
         for (void* q : p->graph_cache) {
             GraphEntry* g = static_cast<GraphEntry*>(q);
             if (g->pr == pr && g->cut == cut && g->fd == fd && g->out[0] == fm && g->out[1] == fmp && g->out[2] == gm &&
@@ -407,7 +416,7 @@ int run_marchenko(mdc_plan* p, mdc_plan* pr, const int* cut, const float* fd, in
             }
         }
         if (!ge) {
-            ge = new GraphEntry{pr, cut, fd, {fm, fmp, gm, gp}, nv, niter, nref, niter_ref, tol, final_h != nullptr};
+            ge = new GraphEntry{pr, {p->scratch_id, pr->scratch_id}, cut, fd, {fm, fmp, gm, gp}, nv, niter, nref, niter_ref, tol, final_h != nullptr};
             ge->S = new Solver();
             init_solver(*ge->S, p, pr, cut, nv, niter, nref, niter_ref, s);
             st = ge->S->alloc(keep_data);

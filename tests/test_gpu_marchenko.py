@@ -256,3 +256,36 @@ def test_redatuming_workload_full_size_two_points():
     print(f"full-size redatuming, 2 points: complex64 {e_plain:.2e}, FP16 + refinement {e_ref:.2e}")
     assert e_plain <= TOL
     assert e_ref <= TOL
+
+
+@pytest.mark.parametrize("storage", ["c64", "c16f"])
+def test_graph_of_a_narrow_solve_after_a_wider_call(storage):
+    """A captured solve holds pointers into the handles' scratch; a wider call moves it, and the repeated solve
+    must not replay the old graph (the freed memory is written over here)."""
+    import paper_2011_11120_gb300 as m
+    nt, n, nf = 128, 90, 20
+    rng = np.random.default_rng(8)
+    G = (rng.standard_normal((nf, n, n)) + 1j * rng.standard_normal((nf, n, n))) * (0.2 / np.sqrt(n))
+    Gt = torch.from_numpy(G.astype(np.complex64)).cuda()
+    op, ref = m.MDC(Gt, nt, 1.0, 1.0, storage=storage), m.MDC(Gt, nt, 1.0, 1.0, storage="c32s")
+    cut = torch.from_numpy(rng.integers(nt // 16, nt // 2, (n, 5)).astype(np.int32)).cuda()
+    fd = torch.from_numpy(rng.standard_normal((nt, n, 5)).astype(np.float32)).cuda()
+    out = [torch.empty_like(fd) for _ in range(4)]
+    m.mdc_set_option(op.h, m.MDC_OPT_GRAPHS, 1)
+
+    def solve():
+        for t in out:
+            t.zero_()
+        m.marchenko_lsqr_refined(op.h, ref.h, cut, fd, 5, 3, 1, 2, 0.0, *out)
+        return [t.clone() for t in out]
+
+    want = solve()
+    for wide in (op, ref):
+        wide.forward(torch.randn((nt, n, 64), device="cuda"))
+        junk = [torch.full((1 << 20,), float("nan"), device="cuda") for _ in range(64)]
+        torch.cuda.synchronize()
+        for a, b in zip(solve(), want):
+            assert torch.equal(a, b)
+        del junk
+    op.close()
+    ref.close()
