@@ -47,7 +47,11 @@ typedef enum {
 /* Storage format of the library-owned kernel copy (Section "Implementing the batch
  * matrix multiplication operator": the kernel streamed once per pass dominates cost). */
 typedef enum {
-    MDC_C64 = 0,    /* complex float32 (the paper's complex64 kernel, Table 1) */
+    /* complex float32 (the paper's complex64 kernel, Table 1).  Passes and deconvolution of 5 or more
+     * columns multiply on tensor cores, at float32 accuracy for kernel and spectrum parts that are zero or
+     * between 2^-110 and 3.38e38 in magnitude: smaller ones lose the bits below 2^-133, larger ones give
+     * infinities or NaN. */
+    MDC_C64 = 0,
     MDC_C16F = 1,   /* complex float16, one float32 scale per (frequency, row) */
     MDC_CBF16 = 2,  /* complex bfloat16, one float32 scale per (frequency, row) */
     MDC_CE4M3 = 3,  /* complex FP8 E4M3, one float32 scale per (frequency, row); tensor-core products

@@ -5,11 +5,12 @@
 //   forward  D[r][n'] = sum_K' G^[r][K'] BT[n'][K'],  K' = 2s + c,  BT[2n] = (Xr, -Xi), BT[2n+1] = (Xi, Xr)
 //   adjoint  D[m][n'] = sum_r G^[r][m] BT[n'][r],     m = 2s + c,   BT[2n] = Yr,        BT[2n+1] = Yi
 // with every float32 factor written as three bfloat16 terms x = x0 + x1 + x2 (each the rounded
-// remainder; the sum is exact for normal values, and bfloat16 has float32's exponent range, so no
-// scaling is needed) and the six products
+// remainder) and the six products
 //   x0 y0  and  x0 y1 + x1 y0 + x1 y1 + x0 y2 + x2 y0
-// (the dropped ones are below 2^-25 of |x y|).  An entry that is not finite makes the outputs it
-// enters NaN or infinite, as in float32.
+// (the dropped ones are below 2^-25 of |x y|).  Nothing is scaled: the sum of the terms is exact for
+// magnitudes from 2^-110 (the last bit of x2 is then bfloat16's smallest subnormal, 2^-133) to 3.38e38
+// (255.5 2^120, where x0 rounds to infinity); smaller values lose what lies below 2^-133, larger finite ones
+// make the outputs they enter NaN or infinite, as an entry that is not finite does.
 //
 // Accuracy.  The tensor core's float32 accumulation truncates, by about 2^-25 of the running sum per
 // MMA, which a long chain adds up (1e-6 over 48 MMAs).  So x0 y0 goes into an accumulator of its own

@@ -54,6 +54,25 @@ def test_c64_tensor_core_products_match_oracle(nr, ns, nf, nv):
     assert rel(yc, omdc.forward_conj_kernel(G, x, 0.004, 400.0)) <= TOL
 
 
+@pytest.mark.parametrize("scale", [2.0 ** -100, 1.0, 2.0 ** 100])
+@pytest.mark.parametrize("nr,ns,nv", [(40, 2100, 16), (2100, 40, 40)])
+def test_sums_of_one_sign_and_range(nr, ns, nv, scale):
+    """Real parts of one sign, so that the accumulators' truncation does not cancel, with kernels near either
+    end of the range.  Each chunk loses at most four times 2^-25 of itself (1.2e-7), and the float32 additions of
+    66 chunk sums at most half an ulp of the running sum each, 2^-25 on average and of either sign: within TOL."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(nr, ns, 4, nv)
+    G = ((np.abs(G.real) - 1j * np.abs(G.imag)) * scale).astype(np.complex64)
+    x, y = (np.abs(x) / scale).astype(np.float32), (np.abs(y) / scale).astype(np.float32)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    op.close()
+    G = G.astype(np.complex128)
+    assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
+    assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
+
+
 def test_c64_tensor_core_wait_limit():
     """A limit the pipeline cannot meet is reported, and the handle works again with the default one.  The kernel
     (0.9 GB) streams from memory: with every SM's ring of loads in flight a tile takes some microseconds."""
