@@ -142,9 +142,10 @@ __global__ void __launch_bounds__(FFT_THREADS, irfft4_ctas(N1 * N2, MODE, FUSE))
             reg_fft<N2, true>(r);
             if (!has0) continue;
             // r[k2] is the sample t = k1 + N1 k2 of the pair
+            const size_t o0 = (size_t)k1 * a.C + c, ostep = (size_t)N1 * a.C;
 #pragma unroll
             for (int k2 = 0; k2 < N2; ++k2) {
-                const size_t o = (size_t)(k1 + N1 * k2) * a.C + c;
+                const size_t o = o0 + k2 * ostep;
                 if constexpr (VEC > 1) {
                     *reinterpret_cast<float2*>(MDC_AT(a.out, o, 2, nx, a.err, 23)) = r[k2];
                 } else {
