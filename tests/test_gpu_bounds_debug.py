@@ -7,8 +7,9 @@ the handle's error flag and the access is skipped, so `mdc_device_status` would 
 (-8).  A child process loads that library (MDC_LIB_DEBUG=1) and runs shapes chosen to leave partial
 tiles everywhere: odd trace counts and column counts, nr != ns, nt from 64 to 4096 (four-step,
 half-length and radix-2 transforms, fused and separate forward transforms), the complex64 GEMV
-(whole-row and chunked), the SIMT GEMM (wide and narrow tiles), FP16 tensor cores and the swapped E4M3
-kernel, a Marchenko solve and an MDD solve.  Every call must report no miss and match the FP64 oracle.
+(whole-row and chunked), its tensor-core GEMM and, with the operand withheld, the SIMT GEMM (wide and narrow
+tiles), FP16 tensor cores (single CTAs and SM pairs) and the swapped E4M3 kernel, a Marchenko solve and an MDD
+solve.  Every call must report no miss and match the FP64 oracle.
 """
 import json
 import os
@@ -45,21 +46,28 @@ cases = [("c64", 64, 37, 29, 20, 1, 1e-5), ("c64", 256, 45, 61, 40, 3, 1e-5),
          ("c64", 512, 33, 27, 100, 20, 1e-5), ("c64", 128, 70, 130, 30, 40, 1e-5),
          ("c64", 2048, 21, 19, 150, 2, 1e-5), ("c64", 4096, 9, 11, 60, 1, 1e-5),
          ("c64", 256, 16, 6200, 4, 1, 1e-5),
+         ("c64 simt", 512, 33, 27, 100, 20, 1e-5), ("c64 simt", 128, 70, 130, 30, 40, 1e-5),
          ("c16f", 128, 130, 70, 5, 16, 4 * U16), ("c16f", 64, 257, 129, 3, 40, 4 * U16),
+         ("c16f", 64, 257, 129, 3, 70, 4 * U16),
          ("ce4m3", 64, 300, 70, 5, 8, 2.0 ** -10)]
 for st, nt, nr, ns, nf, nv, tol in cases:
+    simt, st = st.endswith(" simt"), st.split()[0]
     G = (rng.standard_normal((nf, nr, ns)) + 1j * rng.standard_normal((nf, nr, ns))) / np.sqrt(ns)
     x = rng.standard_normal((nt, ns, nv)).astype(np.float32)
     y = rng.standard_normal((nt, nr, nv)).astype(np.float32)
     op = m.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), nt, 0.004, 400.0, storage=st)
+    if simt:                                        # no room for the operand: 1 MiB of 3 and 5.5
+        m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, 1)
     if st != "c64":
         m.mdc_reserve(op.h, nv)
+    m.mdc_timing(op.h, True)
     yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
     xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
     m.mdc_device_status(op.h)
+    assert st != "c64" or nv < 5 or m.mdc_timing_read(op.h, "tc_prep")[1] == (0 if simt else 2)
     op.close()
     Gq = G if st == "c64" else dequantised(G, st)
-    key = f"{st}-nt{nt}-{nr}x{ns}-nf{nf}-nv{nv}"
+    key = f"{st}{'-simt' if simt else ''}-nt{nt}-{nr}x{ns}-nf{nf}-nv{nv}"
     out[key] = [rel(yg, omdc.forward(Gq, x, 0.004, 400.0)), rel(xg, omdc.adjoint(Gq, y, 0.004, 400.0)), tol]
 
 # Marchenko LSQR (fused forward transforms, window, time reversal) at nt = 512 and 2048

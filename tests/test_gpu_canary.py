@@ -1,6 +1,7 @@
 """GPU: NaN canaries.  Every output buffer is filled with NaN before the call; the call must overwrite
 every element (an element a kernel forgot to write stays NaN), on ragged shapes that leave partial
-tiles in every kernel: GEMV (1-4 columns), SIMT GEMM, tensor cores, the chunked GEMV, the FFT column
+tiles in every kernel: GEMV (1-4 columns), SIMT GEMM (complex64 without its tensor-core operand), tensor
+cores (complex64; 16-bit on single CTAs and on SM pairs), the chunked GEMV, the FFT column
 tails, the Marchenko and MDD solvers.  Inputs are finite, so every correct output is finite.
 """
 import math
@@ -29,7 +30,8 @@ def kernel(nf, nr, ns, seed):
 @pytest.mark.parametrize("nt,nr,ns,nf,nv", [
     (64, 7, 9, 33, 1),          # tiny, every bin
     (128, 130, 70, 40, 3),      # GEMV, ragged rows
-    (256, 65, 201, 60, 9),      # tensor cores / SIMT, ragged columns
+    (256, 65, 201, 60, 9),      # tensor cores and SIMT, ragged columns
+    (64, 140, 70, 30, 67),      # tensor cores on SM pairs, wide SIMT tiles
     (2048, 33, 40, 300, 2),     # half-length transforms
     (64, 29, 6500, 3, 1),       # chunked forward GEMV
 ])
@@ -40,12 +42,15 @@ def test_mdc_outputs_fully_written(storage, nt, nr, ns, nf, nv):
     g.manual_seed(1)
     x = torch.randn((nt, ns, nv), generator=g, device="cuda")
     y = torch.randn((nt, nr, nv), generator=g, device="cuda")
-    for conj in (False, True):
-        yo = nan_like((nt, nr, nv))
-        op.forward(x, out=yo, conj=conj)
-        xo = nan_like((nt, ns, nv))
-        op.adjoint(y, out=xo, conj=conj)
-        assert bool(torch.isfinite(yo).all()) and bool(torch.isfinite(xo).all())
+    for operand_mb in (0, 1) if storage == "c64" and nv >= 5 else (0,):
+        m.mdc_set_option(op.h, m.MDC_OPT_C64_OPERAND_MB, operand_mb)
+        for conj in (False, True):
+            yo = nan_like((nt, nr, nv))
+            op.forward(x, out=yo, conj=conj)
+            xo = nan_like((nt, ns, nv))
+            op.adjoint(y, out=xo, conj=conj)
+            assert bool(torch.isfinite(yo).all()) and bool(torch.isfinite(xo).all())
+        assert (m.mdc_tc_fallback_count(op.h) > 0) == (operand_mb > 0)
     m.mdc_device_status(op.h)
     op.close()
 

@@ -48,7 +48,7 @@ CASES = [
     (1024, 61, 67, 200, 1),
     (4096, 9, 5, 2049, 2),
     (2048, 17, 23, 300, 1),
-    (128, 45, 133, 40, 11),     # GEMV passes over column groups of 4, 4 and 3
+    (128, 45, 133, 40, 11),     # (GEMV groups of 4, 4 and 3: see the products without operand below)
     (2048, 33, 40, 1025, 3),    # every bin of nt = 2048, Nyquist included
     (2048, 9, 14, 1, 6),        # DC only
 ]
@@ -113,6 +113,21 @@ def test_empty_and_bad_arguments(lib):
     out = op.forward(torch.randn((64, 4, 2), device="cuda"))
     assert float(out.abs().max()) == 0.0
     op.close()
+
+
+# without the tensor-core operand (more than 1 MiB here): GEMV passes over column groups of 4 in both
+# directions, in the adjoint alone, and the SIMT GEMM
+@pytest.mark.parametrize("nt,nr,ns,nf,nv", [(256, 65, 200, 64, 8), (128, 45, 133, 40, 11), (512, 150, 129, 100, 64)])
+def test_products_without_operand_match_oracle(lib, nt, nr, ns, nf, nv):
+    G, x, y = rand_case(nt, nr, ns, nf, nv, seed=nt + nv)
+    op = lib.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), nt, 0.004, 400.0)
+    lib.mdc_set_option(op.h, lib.MDC_OPT_C64_OPERAND_MB, 1)
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    assert lib.mdc_tc_fallback_count(op.h) == 2
+    op.close()
+    assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
+    assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
 
 
 @pytest.mark.parametrize("nv,storage", [(1, "c64"), (64, "c64"), (64, "c32s")])
