@@ -109,10 +109,14 @@ def _check(status: int, where: str) -> None:
         raise MDCError(status, where)
 
 
+# The current stream's raw handle without a Stream object per call, where this torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
-        if torch.cuda.is_initialized():              # the raw handle, without a Stream object per call
-            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 

@@ -14,9 +14,8 @@ constexpr int FFT_THREADS = 256;
 // registers over t = n1 * N2 + n2, then the twiddle W_nt^(n2 k1); pass B: for each k1 an
 // N2-point DFT over the N2 consecutive rows k1 * N2 + n2.  Result bin k = k1 + N1 * k2
 // sits in row k1 * N2 + k2.  Four shared-memory sweeps per transform instead of
-// 2 log2(nt) + 1 for radix 2.  Layout: row t of P complex sequences at
-// t * RS + (t / N2) * BP, RS = P + 1 and BP chosen so that both passes spread a warp's
-// 8-byte accesses over distinct bank pairs.
+// 2 log2(nt) + 1 for radix 2.  Layout: row t of P complex sequences at t * P + (t / N2) * BP, BP
+// chosen so that both passes spread a warp's 8-byte accesses over distinct bank pairs.
 
 __host__ __device__ constexpr int brev_bits(int i, int bits) {
     int r = 0;
