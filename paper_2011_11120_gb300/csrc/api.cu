@@ -127,6 +127,11 @@ static int create_plan(mdc_handle* out, const void* G, const double* weights, in
     p->k0 = k0; p->shard = shard;
     p->dt = dt; p->dr = dr; p->storage = storage;
     p->ldg = round_up(ns, G_PITCH_ALIGN);
+    {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
+            p->sms = n;
+    }
     const size_t rowbytes = (size_t)p->ldg * storage_bytes(storage);
     cudaError_t e = cudaMalloc(&p->G, rowbytes * nr * nfmax);
     float* w_d = nullptr;

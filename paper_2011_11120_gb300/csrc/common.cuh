@@ -134,6 +134,7 @@ struct mdc_plan {
     double dt, dr;
     int storage;
     int64_t ldg;                // row pitch of the kernel copy, in complex elements
+    int sms = 148;              // SMs of the device it was created on
     void* G = nullptr;          // library-owned kernel [nf][nr][ldg] in `storage` format
     float* gscale = nullptr;    // [nf][nr] per-row scales (reduced storage), else null
     float2* tw = nullptr;       // [nt/2] e^{-2 pi i j/nt}, then [nt/2] e^{-2 pi i m/(nt/2)} and [nt/2] its

@@ -179,26 +179,57 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_adj_c64(
 // xs[(v * CPV + j) * pitch + i] = X[CPV * i + j][v], so the 32 lanes of a warp, which hold vectors
 // i..i+31, read consecutive shared-memory words for every j and v.
 //
-// A warp walks RB rows at once: RB * U vectors of G in flight per lane, and every X value read from
-// shared memory serves RB rows.  (One row at a time, short rows exposed a memory latency per vector, and
-// four interleaved columns read shared memory eight ways conflicted.)  Bound by HBM on long rows.
-// Complex64, before / now: 1 column on 441^2 x 64 28.9 / 24.5 us; 4 columns on 441^2 x 64 58 / 26 us,
-// 1681^2 x 150 903 / 591 us, 3721^2 x 60 1691 / 1121 us (adjoint 1005 us); 3 columns there 1478 / 1000
-// us; float16, 1 and 4 columns on 3721^2 x 60 583 / 503 and 1667 / 1025 us.  Every lane adds its
-// products in ascending order of the vectors, whatever RB and U.
-// RB and U by measurement on 441^2, 1681^2, 3721 x 841 and 3721^2 kernels.  SHAPE: whole rows of X staged,
-// chunks of it, or whole rows of more than LONG_ROW columns, where one column of complex64 and split
-// FP16 streams best one row at a time (3721^2 x 200: 3.13 ms, two rows at once 3.17 ms; 441^2 x 64: 29
-// us, 25 us).
-enum { ROWS_WHOLE = 0, ROWS_CHUNK = 1, ROWS_LONG = 2 };
-constexpr int LONG_ROW = 2048;
-template <int FMT, int NVC, int SHAPE> struct FwdRows {
-    static constexpr bool H16 = FMT == MDC_C16F || FMT == MDC_CBF16, WIDE4 = SHAPE == ROWS_CHUNK && NVC == 4;
-    static constexpr int RB = SHAPE == ROWS_LONG ? 1
-                              : (H16 && NVC == 1) || ((H16 || FMT == MDC_C64) && WIDE4) ? 4 : 2;      // rows at once
-    static constexpr int U = SHAPE == ROWS_LONG ? 4
-                             : FMT == MDC_C64 ? (WIDE4 ? 1 : 2) : (H16 && NVC > 1) || (FMT == MDC_C32S && NVC == 2) ? 2 : 1;
+// A warp walks RB rows at once, U steps of a row in flight: RB * U vectors of G per lane, and every X value
+// read from shared memory serves RB rows.  (One row at a time, short rows exposed a memory latency per
+// vector, and four interleaved columns read shared memory eight ways conflicted.)  Every lane adds its
+// products in ascending order of the vectors, whatever RB and U, so the choice does not change a bit.
+// Bound by HBM on long rows.  Complex64, before / now: 1 column on 441^2 x 64 28.6 / 24.9 us; 4 columns
+// on 441^2 x 64 57 / 26 us, 1681^2 x 150 903 / 591 us, 3721^2 x 60 1690 / 1130 us (adjoint 1005 us).
+//
+// More rows at once also take more registers, so fewer CTAs fit an SM, and where that makes a small grid's last
+// wave spill over it costs up to a third: 1 column on 1000 x 2000 x 50 (800 CTAs), two rows at once with
+// 5 CTAs per SM 166 us, one row with 6 139 us; split FP16 on 700 x 1700 x 60 (660 CTAs) 129 and 100 us.
+// So each format and column count has two shapes: the wide one is taken if its waves are no more than the
+// narrow one's, or, where that was faster, from `keep` waves on, when the last one counts for little.
+// Shapes by measurement on 24 whole-row and 12 chunked kernels of 25 to 8281 rows and columns (forms tried: 1 x 2,
+// 1 x 4, 2 x 1, 2 x 2, 4 x 1, 4 x 2): against the kernels of one row at a time the time is 0.81 on average and at
+// most 1.06 (a few whole-row kernels of 30 to 150 us).
+struct FwdShape {
+    int rb, u;              // rows at once, steps in flight
+    bool raw = true;        // load the vectors of U steps, then decode; else decode each as it comes
 };
+struct FwdShapes {
+    FwdShape wide, narrow;
+    int keep = 1 << 30;
+};
+constexpr FwdShapes fwd_shapes(int fmt, int nvc, bool chunked) {
+    const bool h16 = fmt == MDC_C16F || fmt == MDC_CBF16;
+    if (chunked) {
+        if (fmt == MDC_C64) {
+            if (nvc == 1) return {{2, 2}, {1, 4}};
+            return nvc == 2 ? FwdShapes{{4, 2}, {4, 2}} : nvc == 3 ? FwdShapes{{2, 2}, {2, 2}} : FwdShapes{{4, 1}, {4, 1}};
+        }
+        if (h16) return nvc == 3 ? FwdShapes{{2, 1}, {2, 1}} : FwdShapes{{4, 1, nvc < 4}, {4, 1, nvc < 4}};
+        if (fmt == MDC_CE4M3)
+            return nvc == 1 ? FwdShapes{{4, 2}, {2, 2}} : nvc == 2 ? FwdShapes{{4, 2}, {4, 2}} : FwdShapes{{4, 1}, {4, 1}};
+        if (nvc == 1) return {{2, 2}, {2, 2}};
+        return nvc == 2 ? FwdShapes{{4, 2}, {2, 2}} : nvc == 3 ? FwdShapes{{2, 1}, {2, 1}} : FwdShapes{{4, 2}, {4, 2}};
+    }
+    if (fmt == MDC_C64) {
+        if (nvc == 1) return {{2, 2}, {1, 4}};
+        return nvc == 2 ? FwdShapes{{4, 2}, {1, 2}} : nvc == 3 ? FwdShapes{{2, 2}, {1, 4}, 3} : FwdShapes{{2, 2}, {2, 2}};
+    }
+    if (h16) {
+        if (nvc == 1) return fmt == MDC_C16F ? FwdShapes{{2, 2}, {1, 4}, 3} : FwdShapes{{4, 1}, {2, 2}};
+        return nvc == 2 ? FwdShapes{{2, 2}, {2, 1}} : nvc == 3 ? FwdShapes{{4, 1}, {2, 1}} : FwdShapes{{2, 1}, {2, 1}};
+    }
+    if (fmt == MDC_CE4M3) {
+        if (nvc == 1 || nvc == 3) return {{4, 1}, {2, 2}};
+        return nvc == 2 ? FwdShapes{{4, 2}, {2, 1}} : FwdShapes{{4, 1}, {2, 1}};
+    }
+    if (nvc == 1) return {{2, 1}, {1, 4}, 3};
+    return nvc == 2 ? FwdShapes{{2, 2}, {2, 1}} : nvc == 3 ? FwdShapes{{2, 2}, {1, 4}, 3} : FwdShapes{{2, 1}, {2, 1}};
+}
 
 // Place of X[CPV * i + j][v] in shared memory: planes (see above), or, for one column of complex64,
 // both values of a vector side by side (one 16-byte read).
@@ -208,7 +239,7 @@ __device__ __forceinline__ int xs_at(int v, int j, int i, int pitch) {
 }
 
 // acc[q][v] += sum over vectors i = i0 + lane, + 32, ... < i1 of row g[q] times X.
-template <int FMT, int NVC, int RB, int U>
+template <int FMT, int NVC, int RB, int U, bool RAW>
 __device__ __forceinline__ void gemv_rows(const uint4* const (&g)[RB], int i0, int i1, int64_t lo, const float2* xs,
                                           int pitch, int xbase, float2 (&acc)[RB][NVC]) {
     constexpr int CPV = Fmt<FMT>::CPV;
@@ -222,20 +253,46 @@ __device__ __forceinline__ void gemv_rows(const uint4* const (&g)[RB], int i0, i
                 for (int q = 0; q < RB; ++q) cfma(acc[q][v], c[q][j], x);
             }
     };
+    constexpr int PL = FMT == MDC_C32S ? 2 : 1;          // planes: the split format's lo plane is added
+    auto load = [&](uint4 (&w)[RB][PL], int i) {
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+            w[q][0] = ld_stream(g[q] + i);
+            if constexpr (PL == 2) w[q][PL - 1] = ld_stream(g[q] + i + lo);
+        }
+    };
+    auto dec = [&](const uint4 (&w)[RB][PL], float2 (&c)[RB][CPV]) {
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+            decode<FMT>(w[q][0], c[q]);
+            if constexpr (PL == 2) {
+                float2 l[CPV];
+                decode<FMT>(w[q][PL - 1], l);
+#pragma unroll
+                for (int j = 0; j < CPV; ++j) c[q][j] = cadd(c[q][j], l[j]);
+            }
+        }
+    };
     int i = i0 + (threadIdx.x & 31);
     for (; i + 32 * (U - 1) < i1; i += 32 * U) {
-        float2 c[U][RB][CPV];
+        uint4 w[U][RB][PL];
+        float2 c[RAW ? 1 : U][RB][CPV];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
+        for (int u = 0; u < U; ++u) {
+            load(w[u], i + 32 * u);
+            if constexpr (!RAW) dec(w[u], c[u]);
+        }
 #pragma unroll
-            for (int q = 0; q < RB; ++q) load_decode<FMT>(g[q], i + 32 * u, lo, c[u][q]);
-#pragma unroll
-        for (int u = 0; u < U; ++u) apply(c[u], i + 32 * u);
+        for (int u = 0; u < U; ++u) {
+            if constexpr (RAW) dec(w[u], c[0]);
+            apply(c[RAW ? 0 : u], i + 32 * u);
+        }
     }
     for (; i < i1; i += 32) {
+        uint4 w[RB][PL];
         float2 c[RB][CPV];
-#pragma unroll
-        for (int q = 0; q < RB; ++q) load_decode<FMT>(g[q], i, lo, c[q]);
+        load(w, i);
+        dec(w, c);
         apply(c, i);
     }
 }
@@ -265,13 +322,12 @@ __device__ __forceinline__ void gemv_rows_store(float2 (&acc)[RB][NVC], const in
     }
 }
 
-template <int FMT, int NVC, int SHAPE>
+template <int FMT, int NVC, int RB, int U, bool RAW>
 __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd(
     const uint4* __restrict__ G, int ldg, int nr, int ns, const float* __restrict__ gscale,
     const float2* __restrict__ X, int ldi, int voff_i,
     float2* __restrict__ Y, int ldo, int voff_o, const int* active, int64_t lo, int* err) {
-    using FR = FwdRows<FMT, NVC, SHAPE>;
-    constexpr int CPV = Fmt<FMT>::CPV, RB = FR::RB, W = GEMV_THREADS / 32;
+    constexpr int CPV = Fmt<FMT>::CPV, W = GEMV_THREADS / 32;
     pdl_wait();
     if (active && *active == 0) return;
     extern __shared__ __align__(16) float2 xs[];   // [NVC][CPV][nvec]
@@ -300,7 +356,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd(
 #pragma unroll
             for (int v = 0; v < NVC; ++v) acc[q][v] = make_float2(0.f, 0.f);
         }
-        gemv_rows<FMT, NVC, RB, FR::U>(g, 0, nvec, lo, xs, nvec, 0, acc);
+        gemv_rows<FMT, NVC, RB, U, RAW>(g, 0, nvec, lo, xs, nvec, 0, acc);
         gemv_rows_store<FMT, NVC, RB>(acc, r, nr, gscale, Y, ldo, voff_o, err);
     }
 }
@@ -416,13 +472,12 @@ struct AdjChunk {
 
 // Forward: the CTA's 32 rows, warp w owning rows r0 + w + 8 q (q < 4) with their partial sums held in
 // registers across chunks.
-template <int FMT, int NVC>
+template <int FMT, int NVC, int RB, int U, bool RAW>
 __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_chunked(
     const uint4* __restrict__ G, int ldg, int nr, int ns, const float* __restrict__ gscale,
     const float2* __restrict__ X, int ldi, int voff_i,
     float2* __restrict__ Y, int ldo, int voff_o, const int* active, int64_t lo, int* err) {
-    using FR = FwdRows<FMT, NVC, ROWS_CHUNK>;
-    constexpr int CPV = Fmt<FMT>::CPV, RB = FR::RB;
+    constexpr int CPV = Fmt<FMT>::CPV;
     constexpr int CHV = FwdChunk<FMT, NVC>::CHV;
     constexpr int W = GEMV_THREADS / 32;
     constexpr int NB = FWD_CHUNK_ROWS / (W * RB);      // batches of RB rows per warp
@@ -461,7 +516,7 @@ __global__ void __launch_bounds__(GEMV_THREADS) gemv_fwd_chunked(
         __syncthreads();
 #pragma unroll
         for (int b = 0; b < NB; ++b)
-            if (r[b][0] < nr) gemv_rows<FMT, NVC, RB, FR::U>(g[b], c0, c1, lo, xs, CHV, c0, acc[b]);       // warp-uniform
+            if (r[b][0] < nr) gemv_rows<FMT, NVC, RB, U, RAW>(g[b], c0, c1, lo, xs, CHV, c0, acc[b]);       // warp-uniform
     }
 #pragma unroll
     for (int b = 0; b < NB; ++b)
@@ -724,33 +779,51 @@ size_t lo_plane_bytes(const mdc_plan* p) {
 }
 int64_t lo_plane_vec(const mdc_plan* p) { return (int64_t)(lo_plane_bytes(p) / 16); }
 
+// CTAs of a GEMV kernel with smem bytes of shared memory that fit an SM (the register limit asked for once).
+template <auto KERN>
+int gemv_ctas_per_sm(size_t smem) {
+    static const int by_regs = [] {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, KERN, GEMV_THREADS, 0) != cudaSuccess) cudaGetLastError();
+        return n > 0 ? n : 1;
+    }();
+    const int by_smem = (int)(228 * 1024 / (smem + 1024));
+    return by_smem < 1 ? 1 : (by_smem < by_regs ? by_smem : by_regs);
+}
+
+// Launch of the wide or the narrow shape (fwd_shapes) for a grid of whole-row or chunked CTAs.
+template <auto WIDE, auto NARROW, int KEEP>
+void gemv_fwd_go(mdc_plan* p, dim3 grid, size_t smem, const float2* in, int ldi, int voff_i, float2* out, int ldo,
+                 int voff_o, cudaStream_t s, const int* active) {
+    bool wide = true;
+    const int n = (int)(grid.x * grid.y);
+    if (WIDE != NARROW && n > p->sms) {
+        auto waves = [&](int per_sm) { return (n + p->sms * per_sm - 1) / (p->sms * per_sm); };
+        const int ww = waves(gemv_ctas_per_sm<WIDE>(smem));
+        wide = ww >= KEEP || ww <= waves(gemv_ctas_per_sm<NARROW>(smem));
+    }
+    static SmemLimit attr[2];
+    attr[wide].ensure(wide ? WIDE : NARROW, 220 * 1024);
+    launch_pdl(wide ? WIDE : NARROW, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G), (int)p->ldg,
+               p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
+}
+
 template <int FMT, int NVC>
 void gemv_fwd_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2* out, int ldo,
                      int voff_o, cudaStream_t s, const int* active) {
     const size_t smem = (size_t)p->ldg * NVC * sizeof(float2);
     if (smem > (size_t)GEMV_STAGE_MAX && gemv_chunk_allowed()) {
         constexpr size_t csmem = (size_t)Fmt<FMT>::CPV * FwdChunk<FMT, NVC>::CHV * NVC * sizeof(float2);
-        dim3 grid((p->nr + FWD_CHUNK_ROWS - 1) / FWD_CHUNK_ROWS, p->nf);
-        launch_pdl(gemv_fwd_chunked<FMT, NVC>, grid, GEMV_THREADS, csmem, s, reinterpret_cast<const uint4*>(p->G),
-                   (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
-                   p->err_flag);
+        constexpr FwdShapes f = fwd_shapes(FMT, NVC, true);
+        gemv_fwd_go<gemv_fwd_chunked<FMT, NVC, f.wide.rb, f.wide.u, f.wide.raw>,
+                    gemv_fwd_chunked<FMT, NVC, f.narrow.rb, f.narrow.u, f.narrow.raw>, f.keep>(
+            p, dim3((p->nr + FWD_CHUNK_ROWS - 1) / FWD_CHUNK_ROWS, p->nf), csmem, in, ldi, voff_i, out, ldo, voff_o, s, active);
         return;
     }
-    dim3 grid((p->nr + FWD_ROWS_PER_CTA - 1) / FWD_ROWS_PER_CTA, p->nf);
-    auto go = [&](auto kern, SmemLimit& attr) {
-        attr.ensure(kern, 220 * 1024);
-        launch_pdl(kern, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G), (int)p->ldg, p->nr,
-                   p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
-    };
-    if constexpr ((FMT == MDC_C64 || FMT == MDC_C32S) && NVC == 1) {
-        if (p->ldg > LONG_ROW) {
-            static SmemLimit attr_long;
-            go(gemv_fwd<FMT, NVC, ROWS_LONG>, attr_long);
-            return;
-        }
-    }
-    static SmemLimit attr;
-    go(gemv_fwd<FMT, NVC, ROWS_WHOLE>, attr);
+    constexpr FwdShapes f = fwd_shapes(FMT, NVC, false);
+    gemv_fwd_go<gemv_fwd<FMT, NVC, f.wide.rb, f.wide.u, f.wide.raw>,
+                gemv_fwd<FMT, NVC, f.narrow.rb, f.narrow.u, f.narrow.raw>, f.keep>(
+        p, dim3((p->nr + FWD_ROWS_PER_CTA - 1) / FWD_ROWS_PER_CTA, p->nf), smem, in, ldi, voff_i, out, ldo, voff_o, s, active);
 }
 
 template <int FMT, int NVC>

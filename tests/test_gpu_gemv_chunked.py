@@ -85,3 +85,21 @@ def test_chunked_and_whole_row_gemv_are_bit_identical(tmp_path):
         res.append(np.load(out))
     assert np.isfinite(res[0]).all()
     assert np.array_equal(res[0], res[1])
+
+
+@pytest.mark.parametrize("storage", ["c64", "c32s", "c16f", "cbf16", "ce4m3"])
+@pytest.mark.parametrize("nr,ns", [(700, 1100), (1000, 400), (1300, 250), (300, 3100)])
+def test_forward_shapes_agree(storage, nr, ns):
+    """The rows a warp takes at once are chosen by the size of the grid; every lane's order of additions is the
+    same, so a kernel's rows give the same bits alone (a small grid) and among many (a grid of a few waves)."""
+    import paper_2011_11120_gb300 as m
+    g = torch.Generator(device="cuda").manual_seed(nr + ns)
+    G = torch.view_as_complex(torch.randn((50, nr, ns, 2), generator=g, device="cuda"))
+    x = torch.randn((128, ns, 4), generator=g, device="cuda")
+    whole = m.MDC(G, 128, 1.0, 1.0, storage=storage)
+    part = m.MDC(G[:, :70].contiguous(), 128, 1.0, 1.0, storage=storage)
+    for nv in (1, 2, 3, 4):
+        xv = x[:, :, :nv].contiguous()
+        assert torch.equal(whole.forward(xv)[:, :70], part.forward(xv))
+    whole.close()
+    part.close()
