@@ -952,6 +952,18 @@ bool launch_product_variant(mdc_plan* p, bool adjoint, const float2* in, int ldi
     return product_simt_or_gemv(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, nullptr, path);
 }
 
+// Complex64 products so small that two launches (operand, GEMM) take longer than the float32 kernels' one or two:
+// adjoints of up to 8 columns on short columns (5 columns, GEMV groups / tensor cores: 25^2 x 40 12 / 14 us,
+// 81^2 x 40 14 / 16, 30 x 1000 x 40 16 / 20; 160^2 x 64 20 / 20, but 1000 x 30 x 40 53 / 28), adjoints of 17 to
+// 32 columns with a reduction of one SIMT step (30 x 1000 x 40 18 / 24), and either on 32^2 or less (24 columns on
+// 25^2 x 40 12 / 16).  Kernels of fewer than 16 rows were not measured.
+static bool c64_small(const mdc_plan* p, bool adjoint, int ncol) {
+    const int64_t entries = (int64_t)p->nr * p->ns;
+    if (p->nr < 16) return false;
+    if (entries <= 1024) return ncol <= 32;
+    return adjoint && entries <= 32768 && (ncol <= 8 ? p->nr <= 160 : (ncol > 16 && ncol <= 32 && p->nr <= 32));
+}
+
 void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int voff_i,
                     float2* out, int ldo, int voff_o, int ncol, cudaStream_t s,
                     const int* active, bool c64_tc) {
@@ -979,7 +991,8 @@ void launch_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int vo
     }
     // complex64: the GEMM runs on tensor cores (same accuracy) wherever its operand exists
     const bool c64_wanted =
-        c64_tc && p->storage == MDC_C64 && (path == PATH_C64_TC || (path == PATH_AUTO && ncol >= C64_TC_MIN));
+        c64_tc && p->storage == MDC_C64 &&
+        (path == PATH_C64_TC || (path == PATH_AUTO && ncol >= C64_TC_MIN && !c64_small(p, adjoint, ncol)));
     if (path == PATH_C64_TC) path = PATH_AUTO;
     if (c64_wanted && tc_c64_ready(p, ncol) &&
         launch_tc_c64(p, adjoint, in, ldi, voff_i, out, ldo, voff_o, ncol, s, active, true))

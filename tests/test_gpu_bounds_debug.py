@@ -43,10 +43,10 @@ rng = np.random.default_rng(5)
 U16 = 2.0 ** -11
 # (storage, nt, nr, ns, nf, nv, tolerance vs the oracle on the stored kernel)
 cases = [("c64", 64, 37, 29, 20, 1, 1e-5), ("c64", 256, 45, 61, 40, 3, 1e-5),
-         ("c64", 512, 33, 27, 100, 20, 1e-5), ("c64", 128, 70, 130, 30, 40, 1e-5),
+         ("c64", 512, 43, 37, 100, 20, 1e-5), ("c64", 128, 70, 130, 30, 40, 1e-5),
          ("c64", 2048, 21, 19, 150, 2, 1e-5), ("c64", 4096, 9, 11, 60, 1, 1e-5),
          ("c64", 256, 16, 6200, 4, 1, 1e-5),
-         ("c64 simt", 512, 33, 27, 100, 20, 1e-5), ("c64 simt", 128, 70, 130, 30, 40, 1e-5),
+         ("c64 simt", 512, 43, 37, 100, 20, 1e-5), ("c64 simt", 128, 70, 130, 30, 40, 1e-5),
          ("c16f", 128, 130, 70, 5, 16, 4 * U16), ("c16f", 64, 257, 129, 3, 40, 4 * U16),
          ("c16f", 64, 257, 129, 3, 70, 4 * U16),
          ("ce4m3", 64, 300, 70, 5, 8, 2.0 ** -10)]

@@ -170,3 +170,21 @@ def test_float32_gemm_matches_oracle(ncol):
     assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
     assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
     assert used == 2
+
+
+# (nr, ns, nv, products on tensor cores): either side of the bounds of the smallest kernels
+@pytest.mark.parametrize("nr,ns,nv,preps", [(32, 32, 5, 0), (33, 32, 24, 2), (32, 32, 33, 2), (160, 204, 8, 1), (161, 204, 8, 2),
+                                            (160, 205, 8, 2), (100, 100, 9, 2), (30, 1000, 17, 1), (30, 1000, 16, 2)])
+def test_smallest_kernels_match_oracle(nr, ns, nv, preps):
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(nr, ns, 5, nv)
+    op = m.MDC(torch.from_numpy(G).cuda(), 64, 0.004, 400.0)
+    m.mdc_timing(op.h, True)
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    got = m.mdc_timing_read(op.h, "tc_prep")[1], m.mdc_tc_fallback_count(op.h)
+    op.close()
+    G = G.astype(np.complex128)
+    assert rel(yg, omdc.forward(G, x, 0.004, 400.0)) <= TOL
+    assert rel(xg, omdc.adjoint(G, y, 0.004, 400.0)) <= TOL
+    assert got == (preps, 0)

@@ -117,7 +117,7 @@ def test_empty_and_bad_arguments(lib):
 
 # without the tensor-core operand (more than 1 MiB here): GEMV passes over column groups of 4 in both
 # directions, in the adjoint alone, and the SIMT GEMM
-@pytest.mark.parametrize("nt,nr,ns,nf,nv", [(256, 65, 200, 64, 8), (128, 45, 133, 40, 11), (512, 150, 129, 100, 64)])
+@pytest.mark.parametrize("nt,nr,ns,nf,nv", [(256, 165, 200, 64, 8), (128, 45, 133, 40, 11), (512, 150, 129, 100, 64)])
 def test_products_without_operand_match_oracle(lib, nt, nr, ns, nf, nv):
     G, x, y = rand_case(nt, nr, ns, nf, nv, seed=nt + nv)
     op = lib.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), nt, 0.004, 400.0)
