@@ -181,10 +181,10 @@ struct LaunchScope {
 // that starts with it may be launched either way, and one launched without the attribute waits for the
 // whole of its predecessors as always.
 //
-// Only launches of up to PDL_MAX_CTAS (four per SM) take the attribute: there the launch latency counts
-// (forward + adjoint on 441^2 x 64, one column: 57.7 -> 48.5 us; Marchenko on it, 10 iterations: 1.69 ->
-// 1.62 ms).  With the attribute on every launch the waiting CTAs of the next kernel took slots from the
-// long GEMV: 3721^2 x 200, one column, 6.34 -> 7.10 ms.
+// Only launches of up to PDL_MAX_CTAS (four per SM) take the attribute: there the launch latency counts (forward +
+// adjoint on 441^2 x 64, one column: 55.6 -> 47.4 us; of 16 columns on 200^2 x 60, 512 samples, 65 -> 54 us).
+// With it on every launch the waiting CTAs of the next kernel took slots from the long GEMV: 3721^2 x 200, one
+// column, 6.34 -> 7.10 ms.  GEMVs take it for the smallest kernels alone (gemv_launch).
 __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

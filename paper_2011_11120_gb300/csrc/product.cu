@@ -779,6 +779,19 @@ size_t lo_plane_bytes(const mdc_plan* p) {
 }
 int64_t lo_plane_vec(const mdc_plan* p) { return (int64_t)(lo_plane_bytes(p) / 16); }
 
+// A GEMV launch starts under its predecessor (launch_pdl) only for kernels of a few megabytes.  CTAs placed while
+// the predecessor still holds part of the SMs are spread unevenly, which lasts as long as they run: adjoint of 1
+// column, complex64, as usual / early: 81^2 x 40 (2 MB) 9.7 / 8.6 us, 900^2 x 20 31 / 31 us, float16 1300^2 x 20 41 / 60
+// us, 8281^2 x 2 219 / 521 us; forward + adjoint of 4 columns on 200^2 x 100 (32 MB) 41 / 45 us.
+constexpr int64_t GEMV_PDL_BYTES = 8 << 20;
+template <typename... P, typename... A>
+void gemv_launch(const mdc_plan* p, void (*kern)(P...), dim3 grid, size_t smem, cudaStream_t s, A&&... args) {
+    if ((int64_t)p->nf * p->nr * p->ldg * storage_bytes(p->storage) <= GEMV_PDL_BYTES)
+        launch_pdl(kern, grid, GEMV_THREADS, smem, s, args...);
+    else
+        kern<<<grid, GEMV_THREADS, smem, s>>>(static_cast<P>(args)...);
+}
+
 // CTAs of a GEMV kernel with smem bytes of shared memory that fit an SM (the register limit asked for once).
 template <auto KERN>
 int gemv_ctas_per_sm(size_t smem) {
@@ -804,7 +817,7 @@ void gemv_fwd_go(mdc_plan* p, dim3 grid, size_t smem, const float2* in, int ldi,
     }
     static SmemLimit attr[2];
     attr[wide].ensure(wide ? WIDE : NARROW, 220 * 1024);
-    launch_pdl(wide ? WIDE : NARROW, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G), (int)p->ldg,
+    gemv_launch(p, wide ? WIDE : NARROW, grid, smem, s, reinterpret_cast<const uint4*>(p->G), (int)p->ldg,
                p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p), p->err_flag);
 }
 
@@ -838,7 +851,7 @@ void gemv_adj_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
         static SmemLimit cattr;
         cattr.ensure(gemv_adj_chunked<FMT, NVC>, 220 * 1024);
         dim3 grid((unsigned)((p->ldg + TILE - 1) / TILE), p->nf);
-        launch_pdl(gemv_adj_chunked<FMT, NVC>, grid, GEMV_THREADS, csmem, s, reinterpret_cast<const uint4*>(p->G),
+        gemv_launch(p, gemv_adj_chunked<FMT, NVC>, grid, csmem, s, reinterpret_cast<const uint4*>(p->G),
                    (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
                    p->err_flag);
         return;
@@ -850,11 +863,11 @@ void gemv_adj_launch(mdc_plan* p, const float2* in, int ldi, int voff_i, float2*
     if constexpr (FMT == MDC_C64) {
         static SmemLimit attr64;
         attr64.ensure(gemv_adj_c64<NVC>, 220 * 1024);
-        launch_pdl(gemv_adj_c64<NVC>, grid, GEMV_THREADS, smem, s, reinterpret_cast<const float4*>(p->G),
+        gemv_launch(p, gemv_adj_c64<NVC>, grid, smem, s, reinterpret_cast<const float4*>(p->G),
                    (int)p->ldg, p->nr, p->ns, in, ldi, voff_i, out, ldo, voff_o, active, p->err_flag);
         return;
     }
-    launch_pdl(gemv_adj<FMT, NVC>, grid, GEMV_THREADS, smem, s, reinterpret_cast<const uint4*>(p->G),
+    gemv_launch(p, gemv_adj<FMT, NVC>, grid, smem, s, reinterpret_cast<const uint4*>(p->G),
                    (int)p->ldg, p->nr, p->ns, p->gscale, in, ldi, voff_i, out, ldo, voff_o, active, lo_plane_vec(p),
                    p->err_flag);
 }
