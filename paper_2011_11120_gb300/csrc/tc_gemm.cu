@@ -14,7 +14,7 @@
 //            Re X'[s][n] = D[2s][2n] + D[2s+1][2n+1], Im X'[s][n] = D[2s][2n+1] - D[2s+1][2n].
 //            A = the SAME G buffer read MN-major (transposed operand); no second copy.
 //
-// 16-bit products of more than 64 columns run on SM pairs (tc_pair_kernel below).  Otherwise one CTA
+// 16-bit products of more than 64 columns over long reductions run on SM pairs (tc_pair_kernel below).  Otherwise one CTA
 // computes a 128 x BN tile of D for one frequency: warp 0 streams A and B
 // tiles with TMA into a ring of 128-byte-swizzled shared-memory stages, warp 1 (one
 // thread) issues tcgen05.mma (M=128, N=BN, K=16, FP32 accumulation in TMEM), warps
@@ -1439,6 +1439,20 @@ bool launch_tc(const CUtensorMap* maps, const TcArgs& a, uint32_t idesc, dim3 gr
     return true;
 }
 
+// Whether SM pairs take a product of gx column tiles and mrows row tiles per frequency in less time than single
+// CTAs.  Long reductions only: a pair saves operand bytes per stage, but starts and leaves at cluster barriers
+// and hands over through the other CTA (float16, 65 to 256 columns, single CTAs = 1: 4 stages of 64, adjoint of
+// 250 x 2000 x 50, 1.11 to 1.14; 8, forward of 2000 x 250 x 50, 1.06 to 1.16; 16, forward of 1300 x 500 x 100, 0.95 to
+// 1.10; 21, its adjoint, 0.86 to 0.97; 27 and 53, 1681^2 x 40, 0.78 to 0.95).  And a wave of pair tiles takes 0.83
+// of one of single tiles (of as many SMs and twice the rows), so row tiles that are one or odd, and last waves,
+// must not cost more (300^2 x 80, forward, two waves instead of one: 1.30).
+constexpr int PR_MIN_STAGES = 20;
+bool pair_pays(int64_t gx, int64_t mrows, int64_t nf, int kstages, int64_t sms) {
+    auto waves = [](int64_t n, int64_t k) { return (n + k - 1) / k; };
+    return kstages >= PR_MIN_STAGES &&
+           5 * waves(gx * ((mrows + 1) / 2) * nf, sms / 2) <= 6 * waves(gx * mrows * nf, sms);
+}
+
 // The SM-pair kernel over (column tiles, row-pair tiles, frequencies); false if no cluster can run.
 template <bool ADJ>
 bool launch_pair(const CUtensorMap* maps, const TcArgs& a, uint32_t idesc, dim3 grid, cudaStream_t s,
@@ -1610,8 +1624,10 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
     const size_t blo = plane * 2;                                          // lo plane of B (bytes)
     // row tiles of the product (kernel rows forward; 2 * ldg interleaved reals adjoint)
     const int mrows = adjoint ? (int)(kp / TC_BM) : (p->nr + TC_BM - 1) / TC_BM;
-    // 256-column tiles of the 16-bit copies run on SM pairs, each CTA loading half of a tile's B rows
-    const bool pair = bn == PR_BN && !split && !e4m3;
+    // 256-column tiles of the 16-bit copies run on SM pairs, each CTA loading half of a tile's B rows, where
+    // that pays
+    const int kstages = adjoint ? (p->nr + TC_BK - 1) / TC_BK : (int)(kp / TC_BK);
+    const bool pair = bn == PR_BN && !split && !e4m3 && pair_pays(rows_pad / bn, mrows, p->nf, kstages, p->sms);
     const int bbox = pair ? bn / 2 : bn;
     bool ok = true;
     const uint64_t ab = e4m3 ? 1 : 2;         // bytes per real of the kernel copy
@@ -1639,7 +1655,7 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
     }
     TcArgs a{};
     a.nf = p->nf;
-    a.kstages = adjoint ? (p->nr + TC_BK - 1) / TC_BK : (int)(kp / TC_BK);
+    a.kstages = kstages;
     a.nout = adjoint ? p->ns : p->nr;
     a.nr = p->nr;
     a.ncol = ncol;
@@ -1680,9 +1696,9 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
         MDC_TC_CASE(32)
         MDC_TC_CASE(64)
         MDC_TC_CASE(128)
-        case 256:                                    // E4M3 (the 16-bit copies run on pairs, split has no 256)
-            launched = adjoint ? launch_tc<true, 256, false, true>(maps, a, idesc, grid, s, active)
-                               : launch_tc<false, 256, false, true>(maps, a, idesc, grid, s, active);
+        case 256:                                    // (split has no 256)
+            if (adjoint) { MDC_TC_LAUNCH(true, 256, false) }
+            else { MDC_TC_LAUNCH(false, 256, false) }
             break;
     }
 #undef MDC_TC_CASE

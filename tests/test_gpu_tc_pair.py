@@ -1,4 +1,4 @@
-"""16-bit products of 65 columns or more, computed by SM pairs (256 x 256 tiles, 128 rows per CTA): parity
+"""16-bit products of 65 columns or more, over long reductions by SM pairs (256 x 256 tiles, 128 rows per CTA): parity
 with the FP64 oracle on the dequantised kernel at the tiles' edges, and the bounded waits.
 
 Tolerance: the spectra are rounded to the 16-bit type after a power-of-two scale, relative error per entry
@@ -18,6 +18,9 @@ pytestmark = pytest.mark.gpu
 # both directions; one and several column tiles with remainders; one reduction slice and many
 CASES = [(256, 128, 3, 128), (100, 60, 4, 65), (257, 129, 3, 127), (255, 127, 3, 130), (129, 400, 2, 256),
          (700, 33, 2, 70)]
+# the same edges with a reduction of 20 stages or more, which pairs take: forward, then adjoint
+LONG = [(256, 600, 3, 128), (100, 620, 4, 65), (257, 577, 3, 127), (255, 700, 3, 130), (129, 900, 2, 256),
+        (1217, 64, 3, 128), (1281, 60, 4, 65), (1300, 129, 3, 127), (1250, 127, 3, 130), (1400, 33, 2, 70)]
 
 
 def problem(nr, ns, nf, nv, nt=64):
@@ -27,11 +30,29 @@ def problem(nr, ns, nf, nv, nt=64):
 
 
 @pytest.mark.parametrize("storage", ["c16f", "cbf16"])
-@pytest.mark.parametrize("nr,ns,nf,nv", CASES)
+@pytest.mark.parametrize("nr,ns,nf,nv", CASES + LONG)
 def test_pair_products_match_oracle(storage, nr, ns, nf, nv):
     import paper_2011_11120_gb300 as m
     G, x, y = problem(nr, ns, nf, nv)
     op = m.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), 64, 0.004, 400.0, storage=storage)
+    yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
+    m.mdc_device_status(op.h)
+    assert m.mdc_tc_fallback_count(op.h) == 0
+    op.close()
+    Gq = dequantised(G, storage)
+    tol = 4 * FORMATS[storage][0]
+    assert rel(yg, omdc.forward(Gq, x, 0.004, 400.0)) <= tol
+    assert rel(xg, omdc.adjoint(Gq, y, 0.004, 400.0)) <= tol
+
+
+@pytest.mark.parametrize("storage", ["c16f", "cbf16"])
+@pytest.mark.parametrize("nr,ns,nf,nv", [(39, 173, 39, 245), (300, 90, 80, 70), (128, 64, 160, 66)])
+def test_single_cta_products_match_oracle(storage, nr, ns, nf, nv):
+    """Shapes that pairs would waste (one row tile, three, with a last wave to spare), in one direction or both."""
+    import paper_2011_11120_gb300 as m
+    G, x, y = problem(nr, ns, nf, nv, nt=512)
+    op = m.MDC(torch.from_numpy(G.astype(np.complex64)).cuda(), 512, 0.004, 400.0, storage=storage)
     yg = op.forward(torch.from_numpy(x).cuda()).cpu().numpy()
     xg = op.adjoint(torch.from_numpy(y).cuda()).cpu().numpy()
     m.mdc_device_status(op.h)
@@ -64,7 +85,7 @@ def test_pair_wait_limit():
     assert rel(yg, omdc.forward(dequantised(G, "c16f"), x, 0.004, 400.0)) <= 4 * FORMATS["c16f"][0]
 
 
-@pytest.mark.parametrize("nr,ns", [(300, 1100), (700, 2300)])
+@pytest.mark.parametrize("nr,ns", [(300, 1100), (700, 2300), (2300, 400)])
 def test_pair_leaves_nothing_behind(nr, ns):
     """Limits around the time of a step, so that waits run out in some pairs and in either CTA of a pair, at any
     step: every launch ends, its status is a timeout or none, and products launched right behind it on the
