@@ -134,12 +134,22 @@ __global__ void __launch_bounds__(FFT_THREADS, irfft4_ctas(N1 * N2, MODE, FUSE))
 
     [[maybe_unused]] const long long nx = (long long)NT * a.C;
     if constexpr (PLAIN) {
+        // Columns that are not in aligned pairs: stored from the registers, each pair is two stores of every
+        // other word of a row.  From nt = 512 on they go out through the tile, a column per thread
+        // (8281 x 255 columns, registers against tile: nt = 1024 4.45 and 3.89 ms, 512 1.64 and 1.52, 256 0.69 and
+        // 0.72, 64 0.225 and 0.240).
+        constexpr bool ROWS = VEC == 1 && NT >= 512;
         for (int task = threadIdx.x; task < P * N1; task += FFT_THREADS) {
             const int k1 = task / P;
             float2 r[N2];
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) r[n2] = z[F::zi(k1 * N2 + n2, j)];
             reg_fft<N2, true>(r);
+            if constexpr (ROWS) {
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) z[F::zi(k1 * N2 + k2, j)] = r[k2];
+                continue;
+            }
             if (!has0) continue;
             // r[k2] is the sample t = k1 + N1 k2 of the pair
             const size_t o0 = (size_t)k1 * a.C + c, ostep = (size_t)N1 * a.C;
@@ -151,6 +161,18 @@ __global__ void __launch_bounds__(FFT_THREADS, irfft4_ctas(N1 * N2, MODE, FUSE))
                 } else {
                     *MDC_AT(a.out, o, 1, nx, a.err, 23) = r[k2].x;
                     if (has1) *MDC_AT(a.out, o + 1, 1, nx, a.err, 24) = r[k2].y;
+                }
+            }
+        }
+        if constexpr (ROWS) {
+            __syncthreads();
+            const int cl = threadIdx.x % CT;
+            if (c0 + cl < a.C) {
+#pragma unroll 8
+                for (int rho = threadIdx.x / CT; rho < NT; rho += FFT_THREADS / CT) {
+                    const int t = (rho % N2) * N1 + rho / N2;
+                    *MDC_AT(a.out, (size_t)t * a.C + c0 + cl, 1, nx, a.err, 24) =
+                        reinterpret_cast<const float*>(z + F::zi(rho, 0))[cl];
                 }
             }
         }
