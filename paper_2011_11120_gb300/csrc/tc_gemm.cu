@@ -1446,11 +1446,21 @@ bool launch_tc(const CUtensorMap* maps, const TcArgs& a, uint32_t idesc, dim3 gr
 // 1.10; 21, its adjoint, 0.86 to 0.97; 27 and 53, 1681^2 x 40, 0.78 to 0.95).  And a wave of pair tiles takes 0.83
 // of one of single tiles (of as many SMs and twice the rows), so row tiles that are one or odd, and last waves,
 // must not cost more (300^2 x 80, forward, two waves instead of one: 1.30).
-constexpr int PR_MIN_STAGES = 20;
-bool pair_pays(int64_t gx, int64_t mrows, int64_t nf, int kstages, int64_t sms) {
+// With several column tiles both kernels keep the tensor cores busy, and a product of more than a millisecond
+// or two runs at the power limit, where pairs gain nothing and leave lower clocks to what follows (dense random
+// kernels, single = 1, in 10^12 operations with the padding: 1.6, forward 1681^2 x 250 of 256 columns, 0.99; 2.3, of
+// 384, 1.03; 5.9, 3721^2 x 200 of 256, 1.01; 11.8, of 512, 1.075; 15.5, 5600^2 x 120 of 512, 1.10).  Adjoints of
+// short reductions gain all the same (27 stages, 3.2: 0.87; 40 stages, 2500^2 x 40 of 900 columns, 0.73), longer
+// ones do not (59 stages, 11.8: 1.07; 88, 15.5: 1.07).  One column tile waits for the kernel's bytes
+// and gains at any size (8281^2 x 160, 128 columns: 0.92 and 0.89).
+constexpr int PR_MIN_STAGES = 20, PR_ADJ_STAGES = 40;
+constexpr int64_t PR_MAX_OPS = 2000000000000;
+bool pair_pays(bool adjoint, int64_t gx, int64_t mrows, int64_t nf, int kstages, int64_t sms) {
     auto waves = [](int64_t n, int64_t k) { return (n + k - 1) / k; };
-    return kstages >= PR_MIN_STAGES &&
-           5 * waves(gx * ((mrows + 1) / 2) * nf, sms / 2) <= 6 * waves(gx * mrows * nf, sms);
+    if (kstages < PR_MIN_STAGES || 5 * waves(gx * ((mrows + 1) / 2) * nf, sms / 2) > 6 * waves(gx * mrows * nf, sms))
+        return false;
+    const int64_t ops = 2 * gx * PR_BN * mrows * TC_BM * nf * kstages * TC_BK;
+    return gx == 1 || ops <= PR_MAX_OPS || (adjoint && kstages <= PR_ADJ_STAGES);
 }
 
 // The SM-pair kernel over (column tiles, row-pair tiles, frequencies); false if no cluster can run.
@@ -1627,7 +1637,7 @@ bool launch_tc_product(mdc_plan* p, bool adjoint, const float2* in, int ldi, int
     // 256-column tiles of the 16-bit copies run on SM pairs, each CTA loading half of a tile's B rows, where
     // that pays
     const int kstages = adjoint ? (p->nr + TC_BK - 1) / TC_BK : (int)(kp / TC_BK);
-    const bool pair = bn == PR_BN && !split && !e4m3 && pair_pays(rows_pad / bn, mrows, p->nf, kstages, p->sms);
+    const bool pair = bn == PR_BN && !split && !e4m3 && pair_pays(adjoint, rows_pad / bn, mrows, p->nf, kstages, p->sms);
     const int bbox = pair ? bn / 2 : bn;
     bool ok = true;
     const uint64_t ab = e4m3 ? 1 : 2;         // bytes per real of the kernel copy
